@@ -431,10 +431,11 @@ __global__ void __launch_bounds__(kAdjThreads) adj_main_kernel(const AdjParams<R
         const bool live = act && q < Nq;
         Real sg[3] = {0, 0, 0};
         if (live) {
-          const int64_t sb = (int64_t)(ep0 + e) * 3 * NqP + q;
-          sg[0] = A.sig[sb];
-          sg[1] = A.sig[sb + NqP];
-          sg[2] = A.sig[sb + 2 * NqP];
+          const int sl = A.qslot[q];
+          const Real* sb = A.sig + ((int64_t)(ep0 + e) * A.nsl + (sl & ~3)) * 3 + (sl & 3);
+          sg[0] = sb[0] * A.eps0_r;
+          sg[1] = sb[4] * A.eps0_r;
+          sg[2] = sb[8] * A.eps0_r;
           Real* zz = ZZ + ((e * NqP + q) * 2 + g) * 6;
 #pragma unroll
           for (int u = 0; u < 3; ++u) {

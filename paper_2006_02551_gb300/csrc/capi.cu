@@ -15,6 +15,7 @@
 #include "../../include/wadg.h"
 #include "kernels.cuh"
 #include "refelem.hpp"
+#include "sym_tables.hpp"
 
 using namespace wadg;
 
@@ -105,6 +106,10 @@ struct wadg_ctx {
   DevPtr q[2], rq, p, rp, geo, geof, fnrm, mat, nbr, code, sig, kap, ops, tabs, verts;
   DevPtr src, srcw, pr_elem, pr_ell, pr_out, obj, tdev, stepdev, flag, tcops, errflag;
   DevPtr stored;     // stored-matrix scheme: per PML element operators
+  // symmetric CUDA-core stage: operator blocks, orbit tables, per-element
+  // geometry, adapted source weights; place of each volume point in a sample block
+  DevPtr symops, symtab, geox, srcws, qslot;
+  SymRule sym;       // symmetry of the volume rule (CUDA-core contexts)
   DevPtr dperm;      // internal -> caller element id (int32), device state exchange
   // caller-owned device memory holding the state buffers (wadg_bind_state)
   void* bound = nullptr;
@@ -254,6 +259,37 @@ std::vector<Real> cvt(const std::vector<double>& a) {
   return std::vector<Real>(a.begin(), a.end());
 }
 
+// groups of four sample places of a CUDA-core context's PML elements
+int sample_groups(const wadg_ctx* ctx) {
+  return ctx->sym.G ? (int)ctx->sym.slots.size() / 4 : (ctx->ref.Nq + 3) / 4;
+}
+
+// tables of the symmetric CUDA-core stage and of the sample order
+template <typename Real>
+wadg_status upload_sym(wadg_ctx* ctx) {
+  const RefOps& R = ctx->ref;
+  ctx->sym = detect_symmetry(R);
+  std::vector<double> ops;
+  std::vector<unsigned char> tab;
+  build_sym_tables(R, ctx->sym, ops, tab);
+  // the kernels copy the table at its largest size for the symmetry
+  const int G = ctx->sym.G;
+  if (G) ops.resize(ops.size() + 2 * (sym_groups(R.N, G) - sample_groups(ctx)) * sym_cp(R.Np, G), 0.0);
+  ops.resize(ops.size() + 4, 0.0);
+  std::vector<Real> hr = cvt<Real>(ops);
+  CK(dalloc(ctx->symops, hr.size() * sizeof(Real)));
+  CK(cudaMemcpy(ctx->symops.p, hr.data(), hr.size() * sizeof(Real), cudaMemcpyHostToDevice));
+  CK(dalloc(ctx->symtab, tab.size()));
+  CK(cudaMemcpy(ctx->symtab.p, tab.data(), tab.size(), cudaMemcpyHostToDevice));
+  std::vector<unsigned char> qs(R.Nq, 0);   // zero-weight points share the first place
+  for (int q = 0; q < R.Nq && !G; ++q) qs[q] = (unsigned char)q;
+  for (int i = (int)ctx->sym.slots.size() - 1; i >= 0; --i)
+    if (ctx->sym.slots[i] >= 0) qs[ctx->sym.slots[i]] = (unsigned char)i;
+  CK(dalloc(ctx->qslot, qs.size()));
+  CK(cudaMemcpy(ctx->qslot.p, qs.data(), qs.size(), cudaMemcpyHostToDevice));
+  return WADG_OK;
+}
+
 template <typename Real>
 wadg_status upload_ops(wadg_ctx* ctx) {
   const RefOps& R = ctx->ref;
@@ -317,8 +353,9 @@ wadg_status upload_ops(wadg_ctx* ctx) {
     for (double v : R.Pq) push(v);
     CK(dalloc(ctx->tcops, tf.size() * 4));
     CK(cudaMemcpy(ctx->tcops.p, tf.data(), tf.size() * 4, cudaMemcpyHostToDevice));
+    return WADG_OK;
   }
-  return WADG_OK;
+  return upload_sym<Real>(ctx);
 }
 
 // Stored-matrix scheme (eqs. 10-13, kappa = 1): per PML element and axis the
@@ -508,6 +545,26 @@ wadg_status rebuild_typed(wadg_ctx* ctx) {
     CK(dalloc(ctx->geof, gf.size() * 4));
     CK(cudaMemcpy(ctx->geof.p, gf.data(), gf.size() * 4, cudaMemcpyHostToDevice));
   }
+  if (!ctx->tc) {   // X = dx/dxi, 1/det X, 1/eps, 1/mu for the symmetric stage
+    std::vector<Real> gx(K * 12);
+    for (int64_t e = 0; e < K; ++e) {
+      const int64_t k = ctx->perm[e];
+      double X[3][3];   // column a: half the edge sum along d/dxi_a
+      for (int d = 0; d < 3; ++d) {
+        double v[4];
+        for (int a = 0; a < 4; ++a) v[a] = ctx->vxyz[3 * ctx->etov[4 * k + a] + d];
+        X[d][0] = 0.25 * (v[0] + v[1] - v[2] - v[3]);
+        X[d][1] = 0.25 * (v[0] - v[1] + v[2] - v[3]);
+        X[d][2] = 0.25 * (v[0] - v[1] - v[2] + v[3]);
+      }
+      for (int i = 0; i < 9; ++i) gx[e * 12 + i] = (Real)X[i / 3][i % 3];
+      gx[e * 12 + 9] = (Real)(-2.0 / ctx->J_u[k]);   // det X = -J / 2
+      gx[e * 12 + 10] = (Real)(ctx->eps_r.empty() ? 1.0 : 1.0 / ctx->eps_r[k]);
+      gx[e * 12 + 11] = (Real)(ctx->mu_r.empty() ? 1.0 : 1.0 / ctx->mu_r[k]);
+    }
+    CK(dalloc(ctx->geox, gx.size() * sizeof(Real)));
+    CK(cudaMemcpy(ctx->geox.p, gx.data(), gx.size() * sizeof(Real), cudaMemcpyHostToDevice));
+  }
   CK(dalloc(ctx->fnrm, fn.size() * sizeof(Real)));
   CK(cudaMemcpy(ctx->fnrm.p, fn.data(), fn.size() * sizeof(Real), cudaMemcpyHostToDevice));
   CK(dalloc(ctx->verts, verts.size() * 8));
@@ -541,11 +598,17 @@ wadg_status rebuild_typed(wadg_ctx* ctx) {
   dfree(ctx->sig);
   dfree(ctx->kap);
   if (ctx->K1 > 0) {
-    std::vector<double> rq(3 * Nq);
-    for (int q = 0; q < Nq; ++q) {
-      rq[3 * q] = ctx->ref.rq[q];
-      rq[3 * q + 1] = ctx->ref.sq[q];
-      rq[3 * q + 2] = ctx->ref.tq[q];
+    // sample places: the volume points in order, or in the groups of four of
+    // a CUDA-core context
+    const bool groups = !ctx->tc;
+    const int ns = groups ? 4 * sample_groups(ctx) : (Nq + 3) & ~3;
+    std::vector<double> rq(3 * (size_t)ns, 2.0);   // 2: padding
+    for (int i = 0; i < ns; ++i) {
+      const int q = groups && ctx->sym.G ? ctx->sym.slots[i] : (i < Nq ? i : -1);
+      if (q < 0) continue;
+      rq[3 * i] = ctx->ref.rq[q];
+      rq[3 * i + 1] = ctx->ref.sq[q];
+      rq[3 * i + 2] = ctx->ref.tq[q];
     }
     double prof[16];
     for (int u = 0; u < 3; ++u) {
@@ -561,10 +624,10 @@ wadg_status rebuild_typed(wadg_ctx* ctx) {
     CK(dalloc(dprof, sizeof prof));
     CK(cudaMemcpy(drq.p, rq.data(), rq.size() * 8, cudaMemcpyHostToDevice));
     CK(cudaMemcpy(dprof.p, prof, sizeof prof, cudaMemcpyHostToDevice));
-    const size_t sb = (size_t)ctx->K1 * 3 * ((Nq + 3) & ~3) * sizeof(Real);
+    const size_t sb = (size_t)ctx->K1 * 3 * ns * sizeof(Real);
     CK(dalloc(ctx->sig, sb));
     if (ctx->kappa) CK(dalloc(ctx->kap, sb));
-    CK((launch_pml_samples<Real>(Nq, (int)ctx->K1, (int)ctx->K0, (const double*)ctx->verts.p,
+    CK((launch_pml_samples<Real>(ns, groups, (int)ctx->K1, (int)ctx->K0, (const double*)ctx->verts.p,
                                  (const double*)drq.p, (const double*)dprof.p,
                                  (Real*)ctx->sig.p, (Real*)ctx->kap.p,
                                  ctx->scheme == WADG_PML_EC, ctx->stream)));
@@ -604,7 +667,7 @@ wadg_status upload_sources(wadg_ctx* ctx) {
   ctx->nsrc = 0;
   ctx->src_ok = false;
   std::vector<SrcDev> sd;
-  std::vector<Real> w;
+  std::vector<Real> w, ws;
   for (const wadg_dipole& d : ctx->src_user) {
     double rst[3];
     int64_t k = locate(ctx, d.x, rst);
@@ -620,15 +683,20 @@ wadg_status upload_sources(wadg_ctx* ctx) {
     s.width = d.width;
     s.amp = d.amplitude;
     sd.push_back(s);
+    std::vector<double> wk(Np);
     for (int i = 0; i < Np; ++i) {  // M_k^{-1} l(r_s) = M^{-1} l / J_k
       double a = 0.0;
       for (int j = 0; j < Np; ++j) a += ctx->ref.Minv[i * Np + j] * ell[j];
-      w.push_back((Real)(a / ctx->J_u[k]));
+      wk[i] = a / ctx->J_u[k];
+      w.push_back((Real)wk[i]);
     }
+    for (double v : sym_adapt(ctx->N, wk)) ws.push_back((Real)v);
   }
   CK(dalloc(ctx->src, sd.size() * sizeof(SrcDev)));
   CK(dalloc(ctx->srcw, w.size() * sizeof(Real)));
+  CK(dalloc(ctx->srcws, ws.size() * sizeof(Real)));
   if (!sd.empty()) {
+    CK(cudaMemcpy(ctx->srcws.p, ws.data(), ws.size() * sizeof(Real), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(ctx->src.p, sd.data(), sd.size() * sizeof(SrcDev), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(ctx->srcw.p, w.data(), w.size() * sizeof(Real), cudaMemcpyHostToDevice));
   }
@@ -708,6 +776,15 @@ StageParams<Real> stage_params(wadg_ctx* ctx, int stage, double dt, double t, bo
   P.t_dev = use_tdev ? (const double*)ctx->tdev.p : nullptr;
   P.eps0 = ctx->has_prof ? ctx->prof.eps0 : 1.0;
   P.alpha = 1.0;
+  if (!ctx->tc) {
+    P.symops = (const Real*)ctx->symops.p;
+    P.symtab = (const unsigned char*)ctx->symtab.p;
+    P.geox = (const Real*)ctx->geox.p;
+    P.src_ws = (const Real*)ctx->srcws.p;
+    P.ngroups = sample_groups(ctx);
+    P.split = sym_split<Real>(ctx->N, pml ? ctx->sym.G : 0, pml && ctx->kappa,
+                              (int64_t)P.n_elem * ctx->nb);
+  }
   P.tcops = ctx->tcops.p;
   P.err = (int*)ctx->errflag.p;
   P.inject = ctx->tc ? (int*)ctx->errflag.p + 1 : nullptr;
@@ -727,7 +804,9 @@ cudaError_t launch_pml_class(wadg_ctx* ctx, const StageParams<Real>& P, cudaStre
       return launch_stage_tc(ctx->N, true, P, ctx->nb, s, ctx->bf16, ctx->qc);
     }
   }
-  return launch_stage<Real>(ctx->N, true, ctx->kappa, P, ctx->nb, s, ctx->qc);
+  // CUDA cores: the symmetric stage, or for a rule without symmetry the dense one
+  if (ctx->sym.G) return launch_sym<Real>(ctx->N, ctx->sym.G, ctx->kappa, P, ctx->nb, s);
+  return launch_stage<Real>(ctx->N, ctx->kappa, P, ctx->nb, s, ctx->qc);
 }
 template <typename Real>
 cudaError_t launch_pml_class(wadg_ctx* ctx, const StageParams<Real>& P) {
@@ -739,7 +818,7 @@ template <typename Real>
 cudaError_t launch_std_class(wadg_ctx* ctx, const StageParams<Real>& P, cudaStream_t s) {
   if constexpr (std::is_same<Real, float>::value)
     if (ctx->tc) return launch_stage_tc(ctx->N, false, P, ctx->nb, s, ctx->bf16, ctx->qc);
-  return launch_stage<Real>(ctx->N, false, false, P, ctx->nb, s);
+  return launch_sym<Real>(ctx->N, 0, false, P, ctx->nb, s);
 }
 
 // one element class of one stage of a context, on stream s, with the device
@@ -770,7 +849,7 @@ wadg_status issue_stage(wadg_ctx* ctx, int stage, double dt, double t, bool use_
     return WADG_OK;
   }
   StageParams<Real> A = stage_params<Real>(ctx, stage, dt, t, use_tdev, false);
-  CK(launch_stage<Real>(ctx->N, false, false, A, ctx->nb, ctx->stream));
+  CK(launch_std_class<Real>(ctx, A, ctx->stream));
   if (ctx->K1 > 0) {
     StageParams<Real> B = stage_params<Real>(ctx, stage, dt, t, use_tdev, true);
     CK(launch_pml_class<Real>(ctx, B));
@@ -796,7 +875,7 @@ wadg_status issue_stage_branches(wadg_ctx* ctx, int stage, double dt) {
     StageParams<Real> B = stage_params<Real>(ctx, stage, dt, 0.0, true, true);
     CK(launch_pml_class<Real>(ctx, B));
     StageParams<Real> A = stage_params<Real>(ctx, stage, dt, 0.0, true, false);
-    CK(launch_stage<Real>(ctx->N, false, false, A, ctx->nb, ctx->aux));
+    CK(launch_std_class<Real>(ctx, A, ctx->aux));
   }
   CK(cudaEventRecord(ctx->ev_join, ctx->aux));
   CK(cudaStreamWaitEvent(ctx->stream, ctx->ev_join, 0));
@@ -1072,6 +1151,8 @@ wadg_status wadg_create(int N, wadg_precision prec, int32_t n_batch, int device,
   if (s == WADG_OK) {
     cudaError_t ce = ctx->rs == 8 ? configure_stage_kernels<double>(N)
                                   : configure_stage_kernels<float>(N);
+    if (ce == cudaSuccess && !ctx->tc)
+      ce = ctx->rs == 8 ? configure_sym_kernels<double>(N) : configure_sym_kernels<float>(N);
     if (ce == cudaSuccess && ctx->tc) ce = configure_tc_kernels(N, ctx->bf16);
     if (ce == cudaSuccess && ctx->tc) ce = configure_tc_rows(N, ctx->bf16);
     if (ce == cudaSuccess)
@@ -1111,7 +1192,8 @@ wadg_status wadg_destroy(wadg_ctx* ctx) {
                     &ctx->nbr, &ctx->code, &ctx->sig, &ctx->kap, &ctx->ops, &ctx->tabs,
                     &ctx->verts, &ctx->src, &ctx->srcw, &ctx->pr_elem, &ctx->pr_ell,
                     &ctx->pr_out, &ctx->obj, &ctx->tdev, &ctx->stepdev, &ctx->flag,
-                    &ctx->tcops, &ctx->errflag, &ctx->stored, &ctx->dperm})
+                    &ctx->tcops, &ctx->errflag, &ctx->stored, &ctx->dperm, &ctx->symops,
+                    &ctx->symtab, &ctx->geox, &ctx->srcws, &ctx->qslot})
     dfree(*d);
   if (ctx->aux) cudaStreamDestroy(ctx->aux);
   if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
@@ -1148,7 +1230,7 @@ wadg_status wadg_set_mesh_periodic(wadg_ctx* ctx, int64_t nv, const double* vxyz
   ctx->ready = false;
   // the point tables refer to the old element order: drop them
   invalidate_graphs(ctx);
-  for (DevPtr* d : {&ctx->src, &ctx->srcw, &ctx->pr_elem, &ctx->pr_ell}) dfree(*d);
+  for (DevPtr* d : {&ctx->src, &ctx->srcw, &ctx->srcws, &ctx->pr_elem, &ctx->pr_ell}) dfree(*d);
   ctx->nsrc = ctx->nprobe = 0;
   ctx->src_ok = ctx->probes_ok = true;
   ctx->K = K;
@@ -1559,12 +1641,11 @@ wadg_status wadg_profile_stage(wadg_ctx* ctx, int reps, double dt, double* ms_ou
       if (ctx->rs == 8) {
         StageParams<double> P = stage_params<double>(ctx, stage, dt, ctx->t, false, cls == 1);
         if (cls == 1) CK(launch_pml_class<double>(ctx, P));
-        else CK(launch_stage<double>(ctx->N, false, false, P, ctx->nb, ctx->stream));
+        else CK(launch_std_class<double>(ctx, P, ctx->stream));
       } else {
         StageParams<float> P = stage_params<float>(ctx, stage, dt, ctx->t, false, cls == 1);
         if (cls == 1) CK(launch_pml_class<float>(ctx, P));
-        else if (ctx->tc) CK(launch_stage_tc(ctx->N, false, P, ctx->nb, ctx->stream, ctx->bf16, ctx->qc));
-        else CK(launch_stage<float>(ctx->N, false, false, P, ctx->nb, ctx->stream));
+        else CK(launch_std_class<float>(ctx, P, ctx->stream));
       }
       CK(cudaEventRecord(ev[2 * cls + 1], ctx->stream));
     }
@@ -1697,6 +1778,9 @@ wadg_status adjoint_typed(wadg_ctx* ctx, int64_t nsteps, double dt, int C, doubl
   A.nsrc = ctx->nsrc; A.src = (const SrcDev*)ctx->src.p; A.src_w = (const Real*)ctx->srcw.p;
   A.dt = dt; A.eps0 = ctx->has_prof ? ctx->prof.eps0 : 1.0; A.alpha = 1.0;
   A.dt_r = (Real)A.dt; A.alpha_r = (Real)A.alpha; A.inv_eps0_r = (Real)(1.0 / A.eps0);
+  A.eps0_r = (Real)A.eps0;
+  A.qslot = (const unsigned char*)ctx->qslot.p;
+  A.nsl = 4 * sample_groups(ctx);
   for (int u = 0; u < 3; ++u) {
     A.sigma_max[u] = ctx->has_prof ? ctx->prof.sigma_max[u] : 0.0;
     A.p_sigma[u] = ctx->has_prof ? ctx->prof.p_sigma[u] : 0.0;
@@ -1722,7 +1806,7 @@ wadg_status adjoint_typed(wadg_ctx* ctx, int64_t nsteps, double dt, int C, doubl
           P.qout = (Real*)b.q.p;
           P.p = (Real*)a.p.p;
           P.pout = (Real*)b.p.p;
-          if (cls == 0) CK(launch_stage<Real>(ctx->N, false, false, P, ctx->nb, ctx->stream));
+          if (cls == 0) CK(launch_std_class<Real>(ctx, P, ctx->stream));
           else CK(launch_pml_class<Real>(ctx, P));
         }
       }
@@ -1945,7 +2029,7 @@ wadg_status noalloc_stage(wadg_ctx* ctx, int stage, double dt, const double* tde
   } else {
     StageParams<Real> A = stage_params<Real>(ctx, stage, dt, 0.0, false, false);
     A.t_dev = tdev;
-    CK(launch_stage<Real>(ctx->N, false, false, A, ctx->nb, ctx->stream));
+    CK(launch_std_class<Real>(ctx, A, ctx->stream));
     if (ctx->K1 > 0) {
       StageParams<Real> B = stage_params<Real>(ctx, stage, dt, 0.0, false, true);
       B.t_dev = tdev;
@@ -2058,7 +2142,7 @@ struct wadg_group {
   bool share = false;      // autotuned: a variant's grid is its share of the GPU (by
                            // algorithmic flops) instead of the whole GPU
   int nblocks = 0;         // all variants
-  struct Item { int c; bool pml; int code; int tile; int64_t tiles; double work; };
+  struct Item { int c; bool pml; int code; int tile; int split; int64_t tiles; double work; };
   std::vector<Item> items;   // sorted by variant code
   // a variant: the items [off, off + n) of one code, its kernel's shared
   // memory and grid, and its block split first[foff .. foff + n]
@@ -2141,6 +2225,10 @@ double item_cost(int N, bool pml) {
 // leave go to the other variants of the stage (parallel graph branches).
 void group_plan(wadg_group* g) {
   g->items.clear();
+  g->variants_ok = true;
+  for (const wadg_ctx* x : g->ctx)
+    if (x->prec != WADG_FP32 || x->qc != 0 || x->sym.G != 2 || x->scheme == WADG_PML_STORED)
+      g->variants_ok = false;
   for (int c = 0; c < (int)g->ctx.size(); ++c) {
     wadg_ctx* x = g->ctx[c];
     for (int cls = 0; cls < 2; ++cls) {
@@ -2151,7 +2239,8 @@ void group_plan(wadg_group* g) {
       it.c = c;
       it.pml = pml;
       it.code = x->N * 4 + (pml ? (x->kappa ? 2 : 1) : 0);
-      const int tmax = g->variants_ok ? group_tile_max(x->N, pml) : 1;
+      it.split = sym_split<float>(x->N, pml ? 2 : 0, pml && x->kappa, ne * x->nb);
+      const int tmax = g->variants_ok ? group_tile_max(it.code, it.split) : 1;
       it.tile = std::max(1, tmax / g->tile_div);
       it.tiles = (ne + it.tile - 1) / it.tile * x->nb;
       it.work = item_cost(x->N, pml) * (double)ne * x->nb;
@@ -2185,7 +2274,7 @@ void group_plan(wadg_group* g) {
     double tot = 0.0;
     for (int j = v.off; j < i; ++j) {
       const auto& it = g->items[j];
-      v.smem = std::max(v.smem, group_smem_bytes(it.code / 4, it.pml, it.tile));
+      v.smem = std::max(v.smem, group_smem_bytes(it.code, it.tile, it.split));
       tot += it.work;
     }
     const int bps = std::max(1, std::min(g->blocks_per_sm, group_blocks_per_sm(v.code, v.smem)));
@@ -2427,11 +2516,6 @@ wadg_status wadg_group_create(int32_t n, wadg_ctx* const* ctxs, wadg_group** out
   }
   wadg_group* g = new wadg_group();
   g->ctx.assign(ctxs, ctxs + n);
-  for (int i = 0; i < n; ++i) {
-    const wadg_ctx* x = ctxs[i];
-    if (x->prec != WADG_FP32 || x->tc || x->qc != 0 || x->scheme == WADG_PML_STORED)
-      g->variants_ok = false;
-  }
   g->device = ctxs[0]->device;
   g->stream = ctxs[0]->stream;
   cudaSetDevice(g->device);

@@ -54,8 +54,7 @@ static cudaError_t launch_one(const StageParams<Real>& P, int nb, cudaStream_t s
 
 template <typename Real, int N>
 static cudaError_t configure_n() {
-  cudaError_t e = configure_one<Real, N, false, false>();
-  if (e == cudaSuccess) e = configure_one<Real, N, true, false>();
+  cudaError_t e = configure_one<Real, N, true, false>();
   if (e == cudaSuccess) e = configure_one<Real, N, true, true>();
   if (e == cudaSuccess) e = configure_one<Real, N, true, false, false, 1>();
   if (e == cudaSuccess) e = configure_one<Real, N, true, true, false, 1>();
@@ -77,9 +76,8 @@ template cudaError_t configure_stage_kernels<double>(int);
 template cudaError_t configure_stage_kernels<float>(int);
 
 template <typename Real, int N>
-static cudaError_t dispatch_pml(bool pml, bool kappa, const StageParams<Real>& P, int nb,
-                                cudaStream_t s, int qc) {
-  if (!pml) return launch_one<Real, N, false, false>(P, nb, s);
+static cudaError_t dispatch_pml(bool kappa, const StageParams<Real>& P, int nb, cudaStream_t s,
+                                int qc) {
   if (qc) {
     if (kappa) return launch_one<Real, N, true, true, false, 1>(P, nb, s);
     return launch_one<Real, N, true, false, false, 1>(P, nb, s);
@@ -89,21 +87,21 @@ static cudaError_t dispatch_pml(bool pml, bool kappa, const StageParams<Real>& P
 }
 
 template <typename Real>
-cudaError_t launch_stage(int N, bool pml, bool kappa, const StageParams<Real>& P, int nb,
-                         cudaStream_t s, int qc) {
+cudaError_t launch_stage(int N, bool kappa, const StageParams<Real>& P, int nb, cudaStream_t s,
+                         int qc) {
   switch (N) {
-    case 1: return dispatch_pml<Real, 1>(pml, kappa, P, nb, s, qc);
-    case 2: return dispatch_pml<Real, 2>(pml, kappa, P, nb, s, qc);
-    case 3: return dispatch_pml<Real, 3>(pml, kappa, P, nb, s, qc);
-    case 4: return dispatch_pml<Real, 4>(pml, kappa, P, nb, s, qc);
-    case 5: return dispatch_pml<Real, 5>(pml, kappa, P, nb, s, qc);
+    case 1: return dispatch_pml<Real, 1>(kappa, P, nb, s, qc);
+    case 2: return dispatch_pml<Real, 2>(kappa, P, nb, s, qc);
+    case 3: return dispatch_pml<Real, 3>(kappa, P, nb, s, qc);
+    case 4: return dispatch_pml<Real, 4>(kappa, P, nb, s, qc);
+    case 5: return dispatch_pml<Real, 5>(kappa, P, nb, s, qc);
     default: return cudaErrorInvalidValue;
   }
 }
-template cudaError_t launch_stage<double>(int, bool, bool, const StageParams<double>&, int,
-                                          cudaStream_t, int);
-template cudaError_t launch_stage<float>(int, bool, bool, const StageParams<float>&, int,
-                                         cudaStream_t, int);
+template cudaError_t launch_stage<double>(int, bool, const StageParams<double>&, int, cudaStream_t,
+                                          int);
+template cudaError_t launch_stage<float>(int, bool, const StageParams<float>&, int, cudaStream_t,
+                                         int);
 
 // ------------------------------------------------------- stored-matrix scheme
 template <typename Real, int N>
@@ -425,19 +423,22 @@ cudaError_t launch_advance(double* t_dev, int64_t* step_dev, double dt, cudaStre
 }
 
 // ---------------------------------------------------------- set-up kernels
-// sigma_u, kappa_u at the quadrature nodes of every PML element, in double.
+// sigma_u, kappa_u at the sample places of every PML element, in double.
 // prof: u0[3], L[3], sigma_max[3], p_sigma[3], kappa_max[3], eps0
 template <typename Real>
-__global__ void pml_samples_kernel(int Nq, int NqP, int K1, int K0, const double* verts,
+__global__ void pml_samples_kernel(int n, bool groups, int K1, int K0, const double* verts,
                                    const double* rq, const double* prof, Real* sig,
                                    Real* kap, bool element_constant) {
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (int64_t)K1 * NqP) return;
-  const int e = (int)(idx / NqP), q = (int)(idx - (int64_t)e * NqP);
-  if (q >= Nq) {   // padding of the quadrature axis
+  if (idx >= (int64_t)K1 * n) return;
+  const int e = (int)(idx / n), q = (int)(idx - (int64_t)e * n);
+  auto at = [&](int u) {
+    return (int64_t)e * 3 * n + (groups ? (q >> 2) * 12 + u * 4 + (q & 3) : u * n + q);
+  };
+  if (rq[q * 3] > 1.0) {   // padding
     for (int u = 0; u < 3; ++u) {
-      sig[((int64_t)e * 3 + u) * NqP + q] = Real(0);
-      if (kap) kap[((int64_t)e * 3 + u) * NqP + q] = Real(1);
+      sig[at(u)] = Real(0);
+      if (kap) kap[at(u)] = Real(1);
     }
     return;
   }
@@ -448,33 +449,32 @@ __global__ void pml_samples_kernel(int Nq, int NqP, int K1, int K0, const double
   const double t = element_constant ? -0.5 : rq[q * 3 + 2];
   const double l0 = -0.5 * (1 + r + s + t), l1 = 0.5 * (1 + r), l2 = 0.5 * (1 + s),
                l3 = 0.5 * (1 + t);
+  const double scale = groups ? 1.0 / prof[15] : 1.0;
   for (int u = 0; u < 3; ++u) {
     const double x = l0 * v[u] + l1 * v[3 + u] + l2 * v[6 + u] + l3 * v[9 + u];
     const double d = (fabs(x) - prof[u]) / prof[3 + u];
     double g = 0.0;
     if (d > 0) g = pow(d, prof[9 + u]);
-    sig[((int64_t)e * 3 + u) * NqP + q] = (Real)(prof[6 + u] * g);
-    if (kap) kap[((int64_t)e * 3 + u) * NqP + q] = (Real)(1.0 + (prof[12 + u] - 1.0) * g);
+    sig[at(u)] = (Real)(prof[6 + u] * g * scale);
+    if (kap) kap[at(u)] = (Real)(1.0 + (prof[12 + u] - 1.0) * g);
   }
 }
 
 template <typename Real>
-cudaError_t launch_pml_samples(int Nq, int K1, int K0, const double* verts, const double* rq,
-                               const double* prof, Real* sig, Real* kap, bool element_constant,
-                               cudaStream_t s) {
-  const int NqP = (Nq + 3) & ~3;
-  const int64_t n = (int64_t)K1 * NqP;
-  if (n == 0) return cudaSuccess;
+cudaError_t launch_pml_samples(int n, bool groups, int K1, int K0, const double* verts,
+                               const double* rq, const double* prof, Real* sig, Real* kap,
+                               bool element_constant, cudaStream_t s) {
+  const int64_t total = (int64_t)K1 * n;
+  if (total == 0) return cudaSuccess;
   const int th = 256;
-  pml_samples_kernel<Real><<<(unsigned)((n + th - 1) / th), th, 0, s>>>(Nq, NqP, K1, K0, verts,
-                                                                       rq, prof, sig, kap,
-                                                                       element_constant);
+  pml_samples_kernel<Real><<<(unsigned)((total + th - 1) / th), th, 0, s>>>(
+      n, groups, K1, K0, verts, rq, prof, sig, kap, element_constant);
   return cudaGetLastError();
 }
-template cudaError_t launch_pml_samples<double>(int, int, int, const double*, const double*,
+template cudaError_t launch_pml_samples<double>(int, bool, int, int, const double*, const double*,
                                                 const double*, double*, double*, bool,
                                                 cudaStream_t);
-template cudaError_t launch_pml_samples<float>(int, int, int, const double*, const double*,
+template cudaError_t launch_pml_samples<float>(int, bool, int, int, const double*, const double*,
                                                const double*, float*, float*, bool, cudaStream_t);
 
 template <typename Real>

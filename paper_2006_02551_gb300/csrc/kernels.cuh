@@ -12,10 +12,15 @@
 //                                  (computed in double on the host)
 //   material mat[e][3]             1/eps, 1/mu, Z = sqrt(mu/eps)
 //   faces    nbr[e][4] (-1: PEC), code[e][4] = neighbour face * 6 + rotation
-//   PML      sig[e'][3][Nq] (and kap[e'][3][Nq])  sigma_u, kappa_u at the
-//            quadrature nodes of each PML element (weight-adjusted scheme;
-//            with element-constant coefficients every node holds the value
-//            at the centroid)
+//            geox[e][12]           CUDA-core contexts: X = dx/dxi [3][3] (xi as in
+//                                  sym_tables.hpp), 1/det X, 1/eps, 1/mu
+//   PML      sig (and kap)  the profile at the quadrature nodes of each PML
+//            element (weight-adjusted scheme; with element-constant
+//            coefficients every node holds the value at the centroid).
+//            CUDA-core contexts: sigma_u/eps0 and kappa_u as
+//            [e'][group][3][4], the nodes in groups of four in the order of
+//            the rule's symmetry (SymRule; its own order without one);
+//            tensor-core contexts: sigma_u as [e'][3][Nq]
 //            stored[e'][3][3][Np][NpP]  stored-matrix scheme: per axis u the
 //            operators M_k^-1 M_k^{b_u}, M_k^-1 M_k^{c_u}, M_k^-1 M_k^{d_u},
 //            transposed (column j of the operator is row j here)
@@ -92,6 +97,13 @@ struct StageParams {
   const double* t_dev;      // device base time (graph replays)
   double eps0;
   double alpha;             // flux upwinding (1 upwind, 0 central)
+  // symmetric CUDA-core stage (sym_body.cuh)
+  const Real* symops;       // operator blocks (SymLayout)
+  const unsigned char* symtab;  // face-node and node orbits
+  const Real* geox;
+  const Real* src_ws;       // [nsrc][Np]: adapted coefficients of src_w
+  int ngroups;              // groups of four volume points
+  int split;                // threads that share a row's groups (sym_split)
   const void* tcops;        // tensor-core operator tables (TF32 path)
   int* err;                 // device error flag (bounded waits that gave up)
   int* inject;              // tensor-core kernels: armed failure-detection request
@@ -117,6 +129,8 @@ struct AdjParams {
   const unsigned char* code;
   const Real* sig;
   const Real* ops;
+  const unsigned char* qslot;   // [Nq]: place of each volume point in a sample block
+  int nsl;                  // sample places per element and axis
   const Real* adj_ops;      // Dr, Ds, Dt [Np][NpP], LIFT [Np][NFP], P_q [Np][NqP], V_q [Nq][NpP]
   const unsigned char* tabs;
   int64_t strideQ, strideP;
@@ -128,7 +142,7 @@ struct AdjParams {
   double sigma_max[3], p_sigma[3];
   Real inv_sigma_max[3], inv_p_sigma[3];   // 1 / sigma_max, 1 / p_sigma (0 where unset)
   // the same scalars rounded once on the host (no per-thread conversion)
-  Real rk_a_r, rk_b_r, dt_r, alpha_r, inv_eps0_r;
+  Real rk_a_r, rk_b_r, dt_r, alpha_r, inv_eps0_r, eps0_r;
 };
 
 struct ProbeParams {
@@ -146,9 +160,21 @@ struct ProbeParams {
 // qc: quadrature class of the PML kernels (quad_capacity)
 template <typename Real>
 cudaError_t configure_stage_kernels(int N);  // once per device, outside graph capture
+// the dense stage of the PML class (volume rules without symmetry)
 template <typename Real>
-cudaError_t launch_stage(int N, bool pml, bool kappa, const StageParams<Real>& P, int nb,
-                         cudaStream_t s, int qc = 0);
+cudaError_t launch_stage(int N, bool kappa, const StageParams<Real>& P, int nb, cudaStream_t s,
+                         int qc = 0);
+// the symmetric stage: G = 0 the non-PML class, 4 or 2 the PML class with a
+// volume rule of that symmetry (SymRule)
+template <typename Real>
+cudaError_t configure_sym_kernels(int N);
+template <typename Real>
+cudaError_t launch_sym(int N, int G, bool kappa, const StageParams<Real>& P, int nb,
+                       cudaStream_t s);
+// threads that share a row's point groups in a class of n elements (times
+// excitations); the same for every launch of the class, whatever its tiles
+template <typename Real>
+int sym_split(int N, int G, bool kappa, int64_t n);
 cudaError_t launch_probes(bool fp64, const ProbeParams& P, cudaStream_t s);
 template <typename Real>
 cudaError_t configure_adjoint_kernels(int N);
@@ -169,10 +195,13 @@ cudaError_t configure_tc_rows(int N, bool bf16);
 cudaError_t launch_pml_tc_rows(int N, const StageParams<float>& P, int nb, cudaStream_t s,
                                bool bf16);
 cudaError_t launch_advance(double* t_dev, int64_t* step_dev, double dt, cudaStream_t s);
+// n sample places per element and axis at the reference points rq [n][3] (a
+// coordinate above 1: padding); groups: [group][3][4] blocks of sigma / eps0,
+// else [3][n] blocks of sigma
 template <typename Real>
-cudaError_t launch_pml_samples(int Nq, int K1, int K0, const double* verts,
-                               const double* rq /*[Nq][3]*/, const double* prof /*16*/,
-                               Real* sig, Real* kap, bool element_constant, cudaStream_t s);
+cudaError_t launch_pml_samples(int n, bool groups, int K1, int K0, const double* verts,
+                               const double* rq, const double* prof /*16*/, Real* sig, Real* kap,
+                               bool element_constant, cudaStream_t s);
 // stored-matrix scheme: the PML class with the per-element operators (3 per
 // axis with kappa = 1: B, C, D; 5 otherwise: B, C, D, K = M^-1 M^{1/kappa},
 // A^-1 = (M^a)^-1 M), and their construction in double precision from the
@@ -188,7 +217,8 @@ template <typename Real>
 cudaError_t launch_stored_ops(int N, int K1, int K0, const double* verts, const double* prof,
                               const double* rh, const double* Ph, const double* Vh, int Nh,
                               bool kappa, Real* out, int* bad, cudaStream_t s);
-// grouped launch (FP32 CUDA-core kernels): item i runs order code[i] / 4 with
+// grouped launch (the symmetric FP32 stage, PML class with a rule of symmetry
+// G = 2, the default one): item i runs order code[i] / 4 with
 // class code[i] % 4 (0 non-PML, 1 PML, 2 PML with kappa); blocks
 // [first[i], first[i+1]) start on item i, and every block takes tiles from
 // counter[i] (zeroed before the launch) until all ntiles[i] are taken, then
@@ -202,11 +232,11 @@ struct GroupParams {
   int nitems;
 };
 cudaError_t configure_group_kernel();
-// dynamic shared memory and largest tile (elements) of one item; threads per
-// block, blocks per SM and launch of the kernel of variant code = N * 4 +
-// (0 non-PML, 1 PML, 2 PML with kappa)
-size_t group_smem_bytes(int N, bool pml, int tile);
-int group_tile_max(int N, bool pml);
+// variant code = N * 4 + (0 non-PML, 1 PML, 2 PML with kappa): dynamic shared
+// memory of an item with `tile` elements per tile, its largest tile, threads
+// per block, blocks per SM and launch
+size_t group_smem_bytes(int code, int tile, int split);
+int group_tile_max(int code, int split);
 int group_threads(int code);
 int group_blocks_per_sm(int code, size_t smem);
 cudaError_t launch_group_stage(int code, const GroupParams& G, int nblocks, size_t smem,

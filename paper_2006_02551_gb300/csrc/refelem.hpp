@@ -50,6 +50,26 @@ bool set_volume_rule(RefOps& o, const std::vector<double>& r, const std::vector<
                      const std::vector<double>& t, const std::vector<double>& w, int pad_to,
                      const char** err);
 
+// Symmetry of a volume rule under the vertex permutations of sym_tables.hpp:
+// G = 4 (V4), 2 (Z2) or 0 (neither).  slots lists the rule's points orbit by
+// orbit in the order of the group's elements (a point that an element fixes
+// appears once for each, -1 pads to a multiple of four).
+struct SymRule {
+  int G = 0;
+  std::vector<int> slots;
+};
+SymRule detect_symmetry(const RefOps& R);
+
+// nodal values -> V4-adapted coefficients (order of Blocks<N, 4>)
+std::vector<double> sym_adapt(int N, const std::vector<double>& f);
+
+// Tables of the symmetric CUDA-core stage (layout: SymLayout): the
+// operators' blocks, and for each node m of face 0 and each element g_y of V4
+// the face-node index [Nfp][4] and the volume node [Nfp][4] of its image,
+// then the nodes of the node orbits and the node nearest the centroid.
+void build_sym_tables(const RefOps& R, const SymRule& S, std::vector<double>& ops,
+                      std::vector<unsigned char>& tabs);
+
 // the six permutations of three face vertices used to encode rotations
 extern const int kFacePerm[6][3];
 // local vertex triples of the four faces (t=-1, s=-1, r+s+t=-1, r=-1)

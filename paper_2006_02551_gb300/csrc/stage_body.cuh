@@ -100,6 +100,12 @@ __device__ __forceinline__ void sts4(double* p, const double* v) {
   *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]);
   *reinterpret_cast<double2*>(p + 2) = make_double2(v[2], v[3]);
 }
+__device__ __forceinline__ void sts2(float* p, const float* v) {
+  *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
+}
+__device__ __forceinline__ void sts2(double* p, const double* v) {
+  *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]);
+}
 __device__ __forceinline__ void lds2(const float* p, float* v) {
   float2 t = *reinterpret_cast<const float2*>(p);
   v[0] = t.x; v[1] = t.y;
@@ -491,7 +497,6 @@ __device__ __forceinline__ void stage_body(const StageParams<Real>& P, unsigned 
 
   // ---- phase 3: V_q of the 12 fields at 4 quadrature points; eq. 9 pointwise
   Real* TZ = U;    // [T][NqP][12]: b VE + c VPE | b VH + c VPH | k^-1 VE - d VPE | k^-1 VH - d VPH
-  const Real ie0 = Real(1) / (Real)P.eps0;
   for (int task = tid; task < ne * NQQ; task += NT) {
     const int e = task / NQQ, qq = task - e * NQQ;
     Real v[12][4];
@@ -512,15 +517,15 @@ __device__ __forceinline__ void stage_body(const StageParams<Real>& P, unsigned 
 #pragma unroll
         for (int n = 0; n < 4; ++n) v[c][n] += w[n] * f[c];
     }
-    const int64_t sb = (int64_t)(ep0 + e) * 3 * NqP + 4 * qq;
+    const int64_t sb = ((int64_t)(ep0 + e) * NQQ + qq) * 12;
     Real sg[3][4], kp[3][4];
     ld4(P.sig + sb, sg[0]);
-    ld4(P.sig + sb + NqP, sg[1]);
-    ld4(P.sig + sb + 2 * NqP, sg[2]);
+    ld4(P.sig + sb + 4, sg[1]);
+    ld4(P.sig + sb + 8, sg[2]);
     if (KAPPA) {
       ld4(P.kap + sb, kp[0]);
-      ld4(P.kap + sb + NqP, kp[1]);
-      ld4(P.kap + sb + 2 * NqP, kp[2]);
+      ld4(P.kap + sb + 4, kp[1]);
+      ld4(P.kap + sb + 8, kp[2]);
     }
 #pragma unroll
     for (int n = 0; n < 4; ++n) {
@@ -532,11 +537,11 @@ __device__ __forceinline__ void stage_body(const StageParams<Real>& P, unsigned 
         const Real ku = KAPPA ? kp[u][n] : Real(1), kv = KAPPA ? kp[vv][n] : Real(1);
         const Real kw = KAPPA ? kp[ww][n] : Real(1);
         const Real su = sg[u][n], sv = sg[vv][n], sw = sg[ww][n];
-        // eq. 9
+        // eq. 9 (the samples are sigma / eps0)
         const Real a = kv * kw / ku;
-        const Real bc = (sv * kw + sw * kv - a * su) / ku * ie0;
-        const Real cc = sv * sw * ie0 * ie0 - bc * su * ie0;
-        const Real dd = su / ku * ie0;
+        const Real bc = (sv * kw + sw * kv - a * su) / ku;
+        const Real cc = sv * sw - bc * su;
+        const Real dd = su / ku;
         const Real ki = Real(1) / ku;
         o[u] = bc * v[u][n] + cc * v[6 + u][n];
         o[3 + u] = bc * v[3 + u][n] + cc * v[9 + u][n];
@@ -619,11 +624,11 @@ __device__ __forceinline__ void stage_body(const StageParams<Real>& P, unsigned 
 #pragma unroll
         for (int n = 0; n < 4; ++n) v[c][n] += w[n] * f[c];
     }
-    const int64_t sb = (int64_t)(ep0 + e) * 3 * NqP + 4 * qq;
+    const int64_t sb = ((int64_t)(ep0 + e) * NQQ + qq) * 12;
     Real kp[3][4];
     ld4(P.kap + sb, kp[0]);
-    ld4(P.kap + sb + NqP, kp[1]);
-    ld4(P.kap + sb + 2 * NqP, kp[2]);
+    ld4(P.kap + sb + 4, kp[1]);
+    ld4(P.kap + sb + 8, kp[2]);
 #pragma unroll
     for (int n = 0; n < 4; ++n) {
       Real* tzo = TZ + (e * NqP + 4 * qq + n) * 12;
