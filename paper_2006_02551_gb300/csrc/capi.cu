@@ -108,8 +108,9 @@ struct wadg_ctx {
   DevPtr stored;     // stored-matrix scheme: per PML element operators
   // symmetric CUDA-core stage: operator blocks, orbit tables, per-element
   // geometry, adapted source weights; place of each volume point in a sample block
-  DevPtr symops, symtab, geox, srcws, qslot;
+  DevPtr symops, symtab, geox, facex, srcws, qslot;
   SymRule sym;       // symmetry of the volume rule (CUDA-core contexts)
+  std::vector<float> symcoef;   // its adapted V_q and P_q in FP32
   DevPtr dperm;      // internal -> caller element id (int32), device state exchange
   // caller-owned device memory holding the state buffers (wadg_bind_state)
   void* bound = nullptr;
@@ -272,9 +273,12 @@ wadg_status upload_sym(wadg_ctx* ctx) {
   std::vector<double> ops;
   std::vector<unsigned char> tab;
   build_sym_tables(R, ctx->sym, ops, tab);
-  // the kernels copy the table at its largest size for the symmetry
   const int G = ctx->sym.G;
-  if (G) ops.resize(ops.size() + 2 * (sym_groups(R.N, G) - sample_groups(ctx)) * sym_cp(R.Np, G), 0.0);
+  ctx->symcoef.clear();
+  if (G)
+    ctx->symcoef.assign(ops.end() - 2 * sample_groups(ctx) * sym_cp(R.N, G), ops.end());
+  // the kernels copy the table at its largest size for the symmetry
+  if (G) ops.resize(ops.size() + 2 * (sym_groups(R.N, G) - sample_groups(ctx)) * sym_cp(R.N, G), 0.0);
   ops.resize(ops.size() + 4, 0.0);
   std::vector<Real> hr = cvt<Real>(ops);
   CK(dalloc(ctx->symops, hr.size() * sizeof(Real)));
@@ -545,7 +549,7 @@ wadg_status rebuild_typed(wadg_ctx* ctx) {
     CK(dalloc(ctx->geof, gf.size() * 4));
     CK(cudaMemcpy(ctx->geof.p, gf.data(), gf.size() * 4, cudaMemcpyHostToDevice));
   }
-  if (!ctx->tc) {   // X = dx/dxi, 1/det X, 1/eps, 1/mu for the symmetric stage
+  if (!ctx->tc) {   // geometry and material of the symmetric stage (geox)
     std::vector<Real> gx(K * 12);
     for (int64_t e = 0; e < K; ++e) {
       const int64_t k = ctx->perm[e];
@@ -557,11 +561,35 @@ wadg_status rebuild_typed(wadg_ctx* ctx) {
         X[d][1] = 0.25 * (v[0] - v[1] + v[2] - v[3]);
         X[d][2] = 0.25 * (v[0] - v[1] - v[2] + v[3]);
       }
-      for (int i = 0; i < 9; ++i) gx[e * 12 + i] = (Real)X[i / 3][i % 3];
+      const double* g = &ctx->metric_u[k * 9];   // grad r, s, t
+      for (int i = 0; i < 9; ++i) {
+        const int a = i / 3, d = i % 3;
+        // grad xi_1 = -(grad s + grad t), and so on
+        gx[e * 12 + i] = sizeof(Real) == 8 ? (Real)X[a][d]
+                                           : (Real)-(g[(a + 1) % 3 * 3 + d] + g[(a + 2) % 3 * 3 + d]);
+      }
       gx[e * 12 + 9] = (Real)(-2.0 / ctx->J_u[k]);   // det X = -J / 2
       gx[e * 12 + 10] = (Real)(ctx->eps_r.empty() ? 1.0 : 1.0 / ctx->eps_r[k]);
       gx[e * 12 + 11] = (Real)(ctx->mu_r.empty() ? 1.0 : 1.0 / ctx->mu_r[k]);
     }
+    std::vector<Real> fx(K * 32);   // the upwind flux's factors per face
+    for (int64_t e = 0; e < K; ++e) {
+      const double Zm = (double)mat[e * 3 + 2];
+      for (int f = 0; f < 4; ++f) {
+        const int nb = nbr[e * 4 + f];
+        const double Zp = nb < 0 ? Zm : (double)mat[nb * 3 + 2];
+        const double w = (double)fn[e * 16 + f * 4 + 3] / (Zm + Zp);
+        Real* o = &fx[e * 32 + f * 8];
+        for (int d = 0; d < 3; ++d) o[d] = fn[e * 16 + f * 4 + d];
+        o[3] = (Real)(Zp * w);
+        o[4] = (Real)w;
+        o[5] = (Real)(Zm * w);
+        o[6] = (Real)(Zm * Zp * w);
+        o[7] = (Real)code[e * 4 + f];
+      }
+    }
+    CK(dalloc(ctx->facex, fx.size() * sizeof(Real)));
+    CK(cudaMemcpy(ctx->facex.p, fx.data(), fx.size() * sizeof(Real), cudaMemcpyHostToDevice));
     CK(dalloc(ctx->geox, gx.size() * sizeof(Real)));
     CK(cudaMemcpy(ctx->geox.p, gx.data(), gx.size() * sizeof(Real), cudaMemcpyHostToDevice));
   }
@@ -780,6 +808,7 @@ StageParams<Real> stage_params(wadg_ctx* ctx, int stage, double dt, double t, bo
     P.symops = (const Real*)ctx->symops.p;
     P.symtab = (const unsigned char*)ctx->symtab.p;
     P.geox = (const Real*)ctx->geox.p;
+    P.facex = (const Real*)ctx->facex.p;
     P.src_ws = (const Real*)ctx->srcws.p;
     P.ngroups = sample_groups(ctx);
     P.split = sym_split<Real>(ctx->N, pml ? ctx->sym.G : 0, pml && ctx->kappa,
@@ -805,7 +834,8 @@ cudaError_t launch_pml_class(wadg_ctx* ctx, const StageParams<Real>& P, cudaStre
     }
   }
   // CUDA cores: the symmetric stage, or for a rule without symmetry the dense one
-  if (ctx->sym.G) return launch_sym<Real>(ctx->N, ctx->sym.G, ctx->kappa, P, ctx->nb, s);
+  if (ctx->sym.G)
+    return launch_sym<Real>(ctx->N, ctx->sym.G, ctx->kappa, P, ctx->symcoef.data(), ctx->nb, s);
   return launch_stage<Real>(ctx->N, ctx->kappa, P, ctx->nb, s, ctx->qc);
 }
 template <typename Real>
@@ -818,7 +848,7 @@ template <typename Real>
 cudaError_t launch_std_class(wadg_ctx* ctx, const StageParams<Real>& P, cudaStream_t s) {
   if constexpr (std::is_same<Real, float>::value)
     if (ctx->tc) return launch_stage_tc(ctx->N, false, P, ctx->nb, s, ctx->bf16, ctx->qc);
-  return launch_sym<Real>(ctx->N, 0, false, P, ctx->nb, s);
+  return launch_sym<Real>(ctx->N, 0, false, P, nullptr, ctx->nb, s);
 }
 
 // one element class of one stage of a context, on stream s, with the device
@@ -1193,7 +1223,7 @@ wadg_status wadg_destroy(wadg_ctx* ctx) {
                     &ctx->verts, &ctx->src, &ctx->srcw, &ctx->pr_elem, &ctx->pr_ell,
                     &ctx->pr_out, &ctx->obj, &ctx->tdev, &ctx->stepdev, &ctx->flag,
                     &ctx->tcops, &ctx->errflag, &ctx->stored, &ctx->dperm, &ctx->symops,
-                    &ctx->symtab, &ctx->geox, &ctx->srcws, &ctx->qslot})
+                    &ctx->symtab, &ctx->geox, &ctx->facex, &ctx->srcws, &ctx->qslot})
     dfree(*d);
   if (ctx->aux) cudaStreamDestroy(ctx->aux);
   if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
@@ -2219,16 +2249,26 @@ double item_cost(int N, bool pml) {
   return f;
 }
 
+// members of the kind that the grouped variant kernels are for
+bool group_variant_members(const wadg_group* g) {
+  for (const wadg_ctx* x : g->ctx)
+    if (x->prec != WADG_FP32 || x->qc != 0 || x->scheme == WADG_PML_STORED) return false;
+  return true;
+}
+
 // work items (sorted by variant), tile sizes, and each variant's grid and
 // block split for the current tuning.  A variant's grid fills the GPU at its
 // own occupancy: its blocks run as long as its tiles last, and the SMs they
 // leave go to the other variants of the stage (parallel graph branches).
 void group_plan(wadg_group* g) {
   g->items.clear();
-  g->variants_ok = true;
-  for (const wadg_ctx* x : g->ctx)
-    if (x->prec != WADG_FP32 || x->qc != 0 || x->sym.G != 2 || x->scheme == WADG_PML_STORED)
-      g->variants_ok = false;
+  g->variants_ok = group_variant_members(g);
+  const wadg_ctx* first_of[6] = {};   // the members of an order share one rule
+  for (const wadg_ctx* x : g->ctx) {
+    const wadg_ctx*& f = first_of[x->N];
+    if (!f) f = x;
+    if (x->sym.G != 2 || x->symcoef != f->symcoef) g->variants_ok = false;
+  }
   for (int c = 0; c < (int)g->ctx.size(); ++c) {
     wadg_ctx* x = g->ctx[c];
     for (int cls = 0; cls < 2; ++cls) {
@@ -2446,7 +2486,9 @@ cudaError_t group_launch(wadg_group* g, int par, int st) {
   for (size_t v = 0; v < nv; ++v) {
     const auto& V = g->vars[v];
     cudaStream_t s = v == 0 || !fork ? g->stream : g->aux[v - 1];
-    e = launch_group_stage(V.code, group_params(g, V, par, st), V.nblocks, V.smem, s);
+    const wadg_ctx* x = g->ctx[g->items[V.off].c];   // the members of an order share one rule
+    e = launch_group_stage(V.code, group_params(g, V, par, st), V.nblocks, V.smem,
+                           x->symcoef.data(), sample_groups(x), s);
     if (e != cudaSuccess) return e;
   }
   for (size_t v = 1; fork && v < nv; ++v) {
@@ -2609,7 +2651,8 @@ wadg_status wadg_group_set_tuning(wadg_group* g, int32_t per_item, int32_t paral
   if (!g) return WADG_EINVAL;
   if (tile_divisor < 1 || tile_divisor > 64 || blocks_per_sm < 1 || blocks_per_sm > 8)
     return gfail(g, WADG_EINVAL, "tile divisor must be 1..64 and blocks per SM 1..8");
-  if (!per_item && !g->variants_ok)
+  // (members whose rules differ, or have no symmetry, run per item all the same)
+  if (!per_item && !group_variant_members(g))
     return gfail(g, WADG_EUNSUPPORTED,
                  "the grouped variant kernels serve FP32 CUDA-core members with the (N+1)^3 "
                  "rule and a weight-adjusted or element-constant PML only");

@@ -21,8 +21,9 @@ using GTile = SymTile<float, N, PML ? 2 : 0, KAPPA>;
 // it, takes that item's tiles from its counter, then moves on to the
 // variant's items that still have tiles
 template <int N, bool PML, bool KAPPA>
-__global__ void __launch_bounds__(kSymThreads, GTile<N, PML, KAPPA>::min_blocks)
-group_stage_kernel(const GroupParams G) {
+__global__ void __launch_bounds__(GTile<N, PML, KAPPA>::NT, GTile<N, PML, KAPPA>::min_blocks)
+group_stage_kernel(const GroupParams G,
+                   const __grid_constant__ SymCoef<GTile<N, PML, KAPPA>::coefs> C) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ StageParams<float> P;
   __shared__ int start;
@@ -43,7 +44,7 @@ group_stage_kernel(const GroupParams G) {
     }
     __syncthreads();
     if (!go) continue;
-    sym_body<float, N, PML ? 2 : 0, KAPPA>(P, smem_raw, 0, 1, G.counter + it);
+    sym_body<float, N, PML ? 2 : 0, KAPPA>(P, C, smem_raw, 0, 1, G.counter + it);
   }
 }
 
@@ -81,36 +82,38 @@ size_t group_smem_bytes(int code, int tile, int split) {
 }
 
 cudaError_t configure_group_kernel() {
-  for (int N = 1; N <= 5; ++N)
+  for (int N = 1; N <= 5; ++N) {
+    cudaError_t e = upload_sym_constants(N);
+    if (e != cudaSuccess) return e;
     for (int v = 0; v < 3; ++v) {
-      cudaError_t e = with_variant(N * 4 + v, [&](auto k, auto t) {
+      e = with_variant(N * 4 + v, [&](auto k, auto t) {
         using ST = decltype(t);
-        const size_t a = ST::bytes(ST::T, ST::S0), b = ST::bytes(ST::tile_max(ST::SS), ST::SS);
         return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)std::max(a, b));
+                                    (int)ST::max_bytes());
       });
       if (e != cudaSuccess) return e;
     }
+  }
   return cudaSuccess;
 }
 
-int group_threads(int) { return kSymThreads; }
+int group_threads(int) { return GTile<1, true, false>::NT; }
 
 int group_blocks_per_sm(int code, size_t smem) {
   int nb = 0;
   cudaError_t e = with_variant(code, [&](auto k, auto) {
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, kSymThreads, smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, (GTile<1, true, false>::NT), smem);
   });
   if (e != cudaSuccess || nb < 1) nb = 1;
   return nb;
 }
 
 cudaError_t launch_group_stage(int code, const GroupParams& G, int nblocks, size_t smem,
-                               cudaStream_t s) {
+                               const float* coef, int ngroups, cudaStream_t s) {
   if (nblocks <= 0 || G.nitems <= 0) return cudaSuccess;
   if (code / 4 < 1 || code / 4 > 5 || code % 4 > 2) return cudaErrorInvalidValue;
-  with_variant(code, [&](auto k, auto) {
-    k<<<nblocks, kSymThreads, smem, s>>>(G);
+  with_variant(code, [&](auto k, auto t) {
+    k<<<nblocks, (GTile<1, true, false>::NT), smem, s>>>(G, sym_coef<decltype(t)>(coef, ngroups));
     return cudaSuccess;
   });
   return cudaGetLastError();

@@ -12,8 +12,12 @@
 //                                  (computed in double on the host)
 //   material mat[e][3]             1/eps, 1/mu, Z = sqrt(mu/eps)
 //   faces    nbr[e][4] (-1: PEC), code[e][4] = neighbour face * 6 + rotation
-//            geox[e][12]           CUDA-core contexts: X = dx/dxi [3][3] (xi as in
-//                                  sym_tables.hpp), 1/det X, 1/eps, 1/mu
+//            facex[e][4][8]        CUDA-core contexts: unit outward normal, Fscale
+//                                  times Z+, 1, Z-, Z- Z+ over Z- + Z+ (the
+//                                  upwind flux's factors), face code
+//            geox[e][12]           CUDA-core contexts, xi as in sym_tables.hpp: FP64 X =
+//                                  dx/dxi [3][3], 1/det X; FP32 grad xi_a [3][3], 0;
+//                                  then 1/eps, 1/mu
 //   PML      sig (and kap)  the profile at the quadrature nodes of each PML
 //            element (weight-adjusted scheme; with element-constant
 //            coefficients every node holds the value at the centroid).
@@ -101,6 +105,7 @@ struct StageParams {
   const Real* symops;       // operator blocks (SymLayout)
   const unsigned char* symtab;  // face-node and node orbits
   const Real* geox;
+  const Real* facex;
   const Real* src_ws;       // [nsrc][Np]: adapted coefficients of src_w
   int ngroups;              // groups of four volume points
   int split;                // threads that share a row's groups (sym_split)
@@ -165,12 +170,13 @@ template <typename Real>
 cudaError_t launch_stage(int N, bool kappa, const StageParams<Real>& P, int nb, cudaStream_t s,
                          int qc = 0);
 // the symmetric stage: G = 0 the non-PML class, 4 or 2 the PML class with a
-// volume rule of that symmetry (SymRule)
+// volume rule of that symmetry (SymRule); coef: the rule's FP32 coefficients in
+// host memory (V_q, then P_q, ngroups x sym_cp(N, G) each), read by the call
 template <typename Real>
 cudaError_t configure_sym_kernels(int N);
 template <typename Real>
-cudaError_t launch_sym(int N, int G, bool kappa, const StageParams<Real>& P, int nb,
-                       cudaStream_t s);
+cudaError_t launch_sym(int N, int G, bool kappa, const StageParams<Real>& P, const float* coef,
+                       int nb, cudaStream_t s);
 // threads that share a row's point groups in a class of n elements (times
 // excitations); the same for every launch of the class, whatever its tiles
 template <typename Real>
@@ -239,8 +245,9 @@ size_t group_smem_bytes(int code, int tile, int split);
 int group_tile_max(int code, int split);
 int group_threads(int code);
 int group_blocks_per_sm(int code, size_t smem);
+// (coef: the variant's rule, as launch_sym's)
 cudaError_t launch_group_stage(int code, const GroupParams& G, int nblocks, size_t smem,
-                               cudaStream_t s);
+                               const float* coef, int ngroups, cudaStream_t s);
 template <typename Real>
 cudaError_t launch_check_finite(const Real* a, int64_t n, int* flag, cudaStream_t s);
 // state exchange between a caller's device array user[nb][K][12][Np] (double,

@@ -70,6 +70,9 @@ std::vector<double> sym_adapt(int N, const std::vector<double>& f);
 void build_sym_tables(const RefOps& R, const SymRule& S, std::vector<double>& ops,
                       std::vector<unsigned char>& tabs);
 
+// the derivative and LIFT blocks of order N in FP32 (SymLayout order), built once
+const std::vector<float>& sym_constants(int N);
+
 // the six permutations of three face vertices used to encode rotations
 extern const int kFacePerm[6][3];
 // local vertex triples of the four faces (t=-1, s=-1, r+s+t=-1, r=-1)

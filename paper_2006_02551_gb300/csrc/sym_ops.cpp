@@ -116,10 +116,10 @@ void tables(const RefOps& R, const SymRule& S, std::vector<double>& ops,
   }
   if (S.G == 0) return;
   const auto TR = S.G == 4 ? T : node_sums_z2<N>();
-  const int G = S.G, CP = sym_cp(Np, G), ng = (int)S.slots.size() / 4, per = 4 / G;
+  const int G = S.G, CP = sym_cp(N, G), ng = (int)S.slots.size() / 4, per = 4 / G;
   const size_t oV = ops.size(), oP = oV + (size_t)ng * CP;
   ops.resize(oP + (size_t)ng * CP, 0.0);
-  auto dim0 = [&](int i) -> int {   // character of adapted index i
+  auto chr = [&](int i) -> int {   // character of adapted index i
     if (G == 4) {
       int x = 0;
       while (x < 3 && i >= B::off(x + 1)) ++x;
@@ -127,12 +127,18 @@ void tables(const RefOps& R, const SymRule& S, std::vector<double>& ops,
     }
     return i >= Blocks<N, 2>::D0 ? 1 : 0;
   };
+  auto place = [&](int o, int i) -> size_t {   // within a group's coefficients
+    const int x = chr(i);
+    using Z = Blocks<N, 2>;
+    return G == 4 ? (size_t)(B::poff(x) + i - B::off(x))
+                  : (size_t)(o * Z::PO + Z::poff(x) + i - Z::off(x));
+  };
   for (int g = 0; g < ng; ++g)
     for (int o = 0; o < per; ++o) {
       const int* sl = &S.slots[4 * g + G * o];
       if (sl[0] < 0) continue;   // padding
       for (int i = 0; i < Np; ++i) {
-        const int x = dim0(i);
+        const int x = chr(i);
         const Signed& ti = TR[i];
         double v = 0.0, w = 0.0;
         for (int y = 0; y < G; ++y) {
@@ -145,8 +151,8 @@ void tables(const RefOps& R, const SymRule& S, std::vector<double>& ops,
           }
         }
         const double n = (double)G * ti.size();
-        ops[oV + (size_t)g * CP + o * Np + i] = v / n;
-        ops[oP + (size_t)g * CP + o * Np + i] = w / n;
+        ops[oV + (size_t)g * CP + place(o, i)] = v / n;
+        ops[oP + (size_t)g * CP + place(o, i)] = w / n;
       }
     }
 }
@@ -227,6 +233,23 @@ void build_sym_tables(const RefOps& R, const SymRule& S, std::vector<double>& op
     case 5: tables<5>(R, S, ops, tabs); break;
     default: break;
   }
+}
+
+const std::vector<float>& sym_constants(int N) {
+  static const std::vector<std::vector<float>> all = [] {
+    std::vector<std::vector<float>> t(6);
+    for (int n = 1; n <= 5; ++n) {
+      RefOps R;
+      const char* err = nullptr;
+      std::vector<double> ops;
+      std::vector<unsigned char> tabs;
+      if (!build_ref_ops(n, R, &err)) continue;
+      build_sym_tables(R, SymRule{}, ops, tabs);
+      t[n].assign(ops.begin(), ops.end());
+    }
+    return t;
+  }();
+  return all[N];
 }
 
 }  // namespace wadg

@@ -98,13 +98,20 @@ struct Blocks {
   static_assert(D0 + (G - 1) * D1 == Np, "block sizes");
   WADG_HD static constexpr int dim(int x) { return x == 0 ? D0 : D1; }
   WADG_HD static constexpr int off(int x) { return x == 0 ? 0 : D0 + (x - 1) * D1; }
+  // offsets with every block padded to an even size (FP32 multiplies pairs)
+  static constexpr int E0 = (D0 + 1) & ~1, E1 = (D1 + 1) & ~1;
+  WADG_HD static constexpr int poff(int x) { return x == 0 ? 0 : E0 + (x - 1) * E1; }
+  static constexpr int PO = E0 + (G - 1) * E1;
+  // coefficients per group of four volume points: of 4 / G point orbits
+  static constexpr int CP = (PO * (4 / G) + 3) & ~3;
 };
 
 // Layout of the operator table of the symmetric stage (in Reals): the
 // derivative blocks by output character x and direction a = 1..3, columns
 // (input value j of character x xor a) of RP(x) rows; the LIFT blocks by x,
 // columns (face-node orbit m) of RP(x) rows; then per group of four volume
-// points (an orbit of V4, or two orbits of Z2) CP coefficients of V_q, and the
+// points (an orbit of V4, or two orbits of Z2) Blocks<N, G>::CP coefficients
+// of V_q (value j of character x of orbit o at o PO + poff(x) + j), and the
 // same of P_q.
 template <int N>
 struct SymLayout {
@@ -125,9 +132,15 @@ struct SymLayout {
   }
   static constexpr int oV = oL + Nfp * (RP0 + 3 * RP1);
 };
-// coefficients per group of four volume points
-WADG_HD constexpr int sym_cp(int Np, int G) { return (Np * (4 / G) + 3) & ~3; }
-
+// Blocks<N, G>::CP
+template <int N>
+WADG_HD constexpr int sym_cp_n(int G) {
+  return G == 4 ? Blocks<N, 4>::CP : Blocks<N, 2>::CP;
+}
+WADG_HD constexpr int sym_cp(int N, int G) {
+  return N == 1 ? sym_cp_n<1>(G) : N == 2 ? sym_cp_n<2>(G) : N == 3 ? sym_cp_n<3>(G)
+       : N == 4 ? sym_cp_n<4>(G) : sym_cp_n<5>(G);
+}
 // largest number of groups of four points that the kernels hold: the compact
 // rules have 1, 5, 6, 13 and 24 orbits under V4 (those of fewer than four
 // points padded); the conical rule of (N + 1)^3 points has N/2 + 1 (rounded
