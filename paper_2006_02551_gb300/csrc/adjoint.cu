@@ -13,7 +13,8 @@
 // launches: adj_lift computes g = Fscale * LIFT^T (mu_E/eps, -mu_H/mu) at the
 // trace nodes of every element (a scratch array), adj_main gathers the own and
 // the neighbour's g to transpose the upwind flux, applies curl^T, V_q^T, P_q^T,
-// and accumulates the parameter derivatives.
+// and accumulates the parameter derivatives.  In FP32 the lift, the non-PML
+// class and the PML class of a symmetric volume rule run sym_adjoint.cu.
 #include "kernels.cuh"
 
 #include <cstdio>
@@ -574,33 +575,44 @@ __global__ void adj_probe_kernel(const Real* q, int64_t strideQ, int nprobe, int
 }
 
 template <typename Real, int N>
-cudaError_t adj_stage_n(const AdjParams<Real>& P, int nb, cudaStream_t s, int qc) {
-  {
+cudaError_t adj_stage_n(const AdjParams<Real>& P, int nb, cudaStream_t s, int qc, int G,
+                        const float* coef) {
+  cudaError_t e;
+  if constexpr (sizeof(Real) == 4) {
+    e = launch_sym_lift(N, P, nb, s);
+  } else {
     dim3 g((P.K + 7) / 8, nb);
     adj_lift_kernel<Real, N><<<g, kAdjThreads, 0, s>>>(P);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    e = cudaGetLastError();
   }
+  if (e != cudaSuccess) return e;
   // non-PML elements, then PML elements
   for (int cls = 0; cls < 2; ++cls) {
     AdjParams<Real> Q = P;
     Q.e_begin = cls == 0 ? 0 : P.K0;
     Q.n_elem = cls == 0 ? P.K0 : P.K - P.K0;
     if (Q.n_elem <= 0) continue;
-    if (cls == 0) {
+    if constexpr (sizeof(Real) == 4) {
+      if (cls == 0 || (G && sym_adjoint_built(N, G))) {
+        e = launch_sym_adjoint(N, cls == 0 ? 0 : G, Q, coef, nb, s);
+        if (e != cudaSuccess) return e;
+        continue;
+      }
+    } else if (cls == 0) {
       using TL = AdjTile<Real, N, false>;
       dim3 g((Q.n_elem + TL::T - 1) / TL::T, nb);
       adj_main_kernel<Real, N, false><<<g, kAdjThreads, TL::smem, s>>>(Q);
-    } else if (qc) {
+    }
+    if (cls == 1 && qc) {
       using TL = AdjTile<Real, N, true, 1>;
       dim3 g((Q.n_elem + TL::T - 1) / TL::T, nb);
       adj_main_kernel<Real, N, true, 1><<<g, kAdjThreads, TL::smem, s>>>(Q);
-    } else {
+    } else if (cls == 1) {
       using TL = AdjTile<Real, N, true>;
       dim3 g((Q.n_elem + TL::T - 1) / TL::T, nb);
       adj_main_kernel<Real, N, true><<<g, kAdjThreads, TL::smem, s>>>(Q);
     }
-    cudaError_t e = cudaGetLastError();
+    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -608,9 +620,13 @@ cudaError_t adj_stage_n(const AdjParams<Real>& P, int nb, cudaStream_t s, int qc
 
 template <typename Real, int N>
 cudaError_t adj_configure_n() {
-  cudaError_t e = cudaFuncSetAttribute(adj_main_kernel<Real, N, false>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)AdjTile<Real, N, false>::smem);
+  cudaError_t e = cudaSuccess;
+  if constexpr (sizeof(Real) == 4)
+    e = configure_sym_adjoint(N);
+  else
+    e = cudaFuncSetAttribute(adj_main_kernel<Real, N, false>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)AdjTile<Real, N, false>::smem);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(adj_main_kernel<Real, N, true>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -639,21 +655,21 @@ template cudaError_t configure_adjoint_kernels<double>(int);
 template cudaError_t configure_adjoint_kernels<float>(int);
 
 template <typename Real>
-cudaError_t launch_adjoint_stage(int N, const AdjParams<Real>& P, int nb, cudaStream_t s,
-                                 int qc) {
+cudaError_t launch_adjoint_stage(int N, const AdjParams<Real>& P, int nb, cudaStream_t s, int qc,
+                                 int G, const float* coef) {
   switch (N) {
-    case 1: return adj_stage_n<Real, 1>(P, nb, s, qc);
-    case 2: return adj_stage_n<Real, 2>(P, nb, s, qc);
-    case 3: return adj_stage_n<Real, 3>(P, nb, s, qc);
-    case 4: return adj_stage_n<Real, 4>(P, nb, s, qc);
-    case 5: return adj_stage_n<Real, 5>(P, nb, s, qc);
+    case 1: return adj_stage_n<Real, 1>(P, nb, s, qc, G, coef);
+    case 2: return adj_stage_n<Real, 2>(P, nb, s, qc, G, coef);
+    case 3: return adj_stage_n<Real, 3>(P, nb, s, qc, G, coef);
+    case 4: return adj_stage_n<Real, 4>(P, nb, s, qc, G, coef);
+    case 5: return adj_stage_n<Real, 5>(P, nb, s, qc, G, coef);
     default: return cudaErrorInvalidValue;
   }
 }
 template cudaError_t launch_adjoint_stage<double>(int, const AdjParams<double>&, int, cudaStream_t,
-                                                  int);
+                                                  int, int, const float*);
 template cudaError_t launch_adjoint_stage<float>(int, const AdjParams<float>&, int, cudaStream_t,
-                                                 int);
+                                                 int, int, const float*);
 
 template <typename Real>
 cudaError_t launch_adjoint_probes(const Real* q, int64_t strideQ, int nprobe, int nb, int Np,

@@ -108,7 +108,7 @@ struct wadg_ctx {
   DevPtr stored;     // stored-matrix scheme: per PML element operators
   // symmetric CUDA-core stage: operator blocks, orbit tables, per-element
   // geometry, adapted source weights; place of each volume point in a sample block
-  DevPtr symops, symtab, geox, facex, srcws, qslot;
+  DevPtr symops, symadj, symtab, geox, facex, srcws, qslot;
   SymRule sym;       // symmetry of the volume rule (CUDA-core contexts)
   std::vector<float> symcoef;   // its adapted V_q and P_q in FP32
   DevPtr dperm;      // internal -> caller element id (int32), device state exchange
@@ -283,6 +283,11 @@ wadg_status upload_sym(wadg_ctx* ctx) {
   std::vector<Real> hr = cvt<Real>(ops);
   CK(dalloc(ctx->symops, hr.size() * sizeof(Real)));
   CK(cudaMemcpy(ctx->symops.p, hr.data(), hr.size() * sizeof(Real), cudaMemcpyHostToDevice));
+  if (sizeof(Real) == 4) {   // the adjoint's transposed blocks
+    const std::vector<float> tr = sym_transposed(R.N, ops);
+    CK(dalloc(ctx->symadj, tr.size() * 4));
+    CK(cudaMemcpy(ctx->symadj.p, tr.data(), tr.size() * 4, cudaMemcpyHostToDevice));
+  }
   CK(dalloc(ctx->symtab, tab.size()));
   CK(cudaMemcpy(ctx->symtab.p, tab.data(), tab.size(), cudaMemcpyHostToDevice));
   std::vector<unsigned char> qs(R.Nq, 0);   // zero-weight points share the first place
@@ -549,50 +554,6 @@ wadg_status rebuild_typed(wadg_ctx* ctx) {
     CK(dalloc(ctx->geof, gf.size() * 4));
     CK(cudaMemcpy(ctx->geof.p, gf.data(), gf.size() * 4, cudaMemcpyHostToDevice));
   }
-  if (!ctx->tc) {   // geometry and material of the symmetric stage (geox)
-    std::vector<Real> gx(K * 12);
-    for (int64_t e = 0; e < K; ++e) {
-      const int64_t k = ctx->perm[e];
-      double X[3][3];   // column a: half the edge sum along d/dxi_a
-      for (int d = 0; d < 3; ++d) {
-        double v[4];
-        for (int a = 0; a < 4; ++a) v[a] = ctx->vxyz[3 * ctx->etov[4 * k + a] + d];
-        X[d][0] = 0.25 * (v[0] + v[1] - v[2] - v[3]);
-        X[d][1] = 0.25 * (v[0] - v[1] + v[2] - v[3]);
-        X[d][2] = 0.25 * (v[0] - v[1] - v[2] + v[3]);
-      }
-      const double* g = &ctx->metric_u[k * 9];   // grad r, s, t
-      for (int i = 0; i < 9; ++i) {
-        const int a = i / 3, d = i % 3;
-        // grad xi_1 = -(grad s + grad t), and so on
-        gx[e * 12 + i] = sizeof(Real) == 8 ? (Real)X[a][d]
-                                           : (Real)-(g[(a + 1) % 3 * 3 + d] + g[(a + 2) % 3 * 3 + d]);
-      }
-      gx[e * 12 + 9] = (Real)(-2.0 / ctx->J_u[k]);   // det X = -J / 2
-      gx[e * 12 + 10] = (Real)(ctx->eps_r.empty() ? 1.0 : 1.0 / ctx->eps_r[k]);
-      gx[e * 12 + 11] = (Real)(ctx->mu_r.empty() ? 1.0 : 1.0 / ctx->mu_r[k]);
-    }
-    std::vector<Real> fx(K * 32);   // the upwind flux's factors per face
-    for (int64_t e = 0; e < K; ++e) {
-      const double Zm = (double)mat[e * 3 + 2];
-      for (int f = 0; f < 4; ++f) {
-        const int nb = nbr[e * 4 + f];
-        const double Zp = nb < 0 ? Zm : (double)mat[nb * 3 + 2];
-        const double w = (double)fn[e * 16 + f * 4 + 3] / (Zm + Zp);
-        Real* o = &fx[e * 32 + f * 8];
-        for (int d = 0; d < 3; ++d) o[d] = fn[e * 16 + f * 4 + d];
-        o[3] = (Real)(Zp * w);
-        o[4] = (Real)w;
-        o[5] = (Real)(Zm * w);
-        o[6] = (Real)(Zm * Zp * w);
-        o[7] = (Real)code[e * 4 + f];
-      }
-    }
-    CK(dalloc(ctx->facex, fx.size() * sizeof(Real)));
-    CK(cudaMemcpy(ctx->facex.p, fx.data(), fx.size() * sizeof(Real), cudaMemcpyHostToDevice));
-    CK(dalloc(ctx->geox, gx.size() * sizeof(Real)));
-    CK(cudaMemcpy(ctx->geox.p, gx.data(), gx.size() * sizeof(Real), cudaMemcpyHostToDevice));
-  }
   CK(dalloc(ctx->fnrm, fn.size() * sizeof(Real)));
   CK(cudaMemcpy(ctx->fnrm.p, fn.data(), fn.size() * sizeof(Real), cudaMemcpyHostToDevice));
   CK(dalloc(ctx->verts, verts.size() * 8));
@@ -603,6 +564,14 @@ wadg_status rebuild_typed(wadg_ctx* ctx) {
   CK(cudaMemcpy(ctx->nbr.p, nbr.data(), nbr.size() * 4, cudaMemcpyHostToDevice));
   CK(dalloc(ctx->code, code.size()));
   CK(cudaMemcpy(ctx->code.p, code.data(), code.size(), cudaMemcpyHostToDevice));
+  if (!ctx->tc) {   // geometry, material and face factors of the symmetric stage
+    CK(dalloc(ctx->facex, (size_t)K * 32 * sizeof(Real)));
+    CK(dalloc(ctx->geox, (size_t)K * 12 * sizeof(Real)));
+    CK((launch_sym_geometry<Real>(K, (const double*)ctx->geo.p, (const double*)ctx->verts.p,
+                                  (const Real*)ctx->fnrm.p, (const Real*)ctx->mat.p,
+                                  (const int*)ctx->nbr.p, (const unsigned char*)ctx->code.p,
+                                  (Real*)ctx->facex.p, (Real*)ctx->geox.p, ctx->stream)));
+  }
   {  // internal -> caller element id, for the device state exchange
     std::vector<int> pm(K);
     for (int64_t e = 0; e < K; ++e) pm[e] = (int)ctx->perm[e];
@@ -1222,7 +1191,7 @@ wadg_status wadg_destroy(wadg_ctx* ctx) {
                     &ctx->nbr, &ctx->code, &ctx->sig, &ctx->kap, &ctx->ops, &ctx->tabs,
                     &ctx->verts, &ctx->src, &ctx->srcw, &ctx->pr_elem, &ctx->pr_ell,
                     &ctx->pr_out, &ctx->obj, &ctx->tdev, &ctx->stepdev, &ctx->flag,
-                    &ctx->tcops, &ctx->errflag, &ctx->stored, &ctx->dperm, &ctx->symops,
+                    &ctx->tcops, &ctx->errflag, &ctx->stored, &ctx->dperm, &ctx->symops, &ctx->symadj,
                     &ctx->symtab, &ctx->geox, &ctx->facex, &ctx->srcws, &ctx->qslot})
     dfree(*d);
   if (ctx->aux) cudaStreamDestroy(ctx->aux);
@@ -1704,14 +1673,26 @@ struct StateBuf {
   DevPtr q, p;
 };
 
-wadg_status alloc_state(wadg_ctx* ctx, StateBuf& b) {
-  CK(dalloc(b.q, ctx->q[0].bytes));
-  CK(dalloc(b.p, ctx->p.bytes));
+// n states in one allocation (a call of the adjoint keeps hundreds: one
+// cudaMalloc and cudaFree each cost more than a stage); each block is followed
+// by kSlack spare bytes and starts on a 256-byte boundary
+wadg_status alloc_states(wadg_ctx* ctx, DevPtr& slab, const std::vector<StateBuf*>& b) {
+  auto room = [](size_t n) { return n ? (n + kSlack + 255) & ~size_t(255) : 0; };
+  const size_t qb = ctx->q[0].bytes, pb = ctx->p.bytes, one = room(qb) + room(pb);
+  CK(dalloc(slab, one * b.size()));
+  unsigned char* at = static_cast<unsigned char*>(slab.p);
+  for (StateBuf* x : b) {
+    x->q.p = at;
+    x->q.bytes = qb;
+    x->q.borrowed = true;
+    if (pb) {
+      x->p.p = at + room(qb);
+      x->p.bytes = pb;
+      x->p.borrowed = true;
+    }
+    at += one;
+  }
   return WADG_OK;
-}
-void free_state(StateBuf& b) {
-  dfree(b.q);
-  dfree(b.p);
 }
 wadg_status save_state(wadg_ctx* ctx, StateBuf& b) {
   CK(cudaMemcpyAsync(b.q.p, ctx->q[ctx->cur].p, b.q.bytes, cudaMemcpyDeviceToDevice, ctx->stream));
@@ -1738,19 +1719,21 @@ wadg_status adjoint_typed(wadg_ctx* ctx, int64_t nsteps, double dt, int C, doubl
   // is recomputed, sin[5k + i - 1] = input of stage i of step k (i = 0, k = 0
   // is the checkpoint itself), sin[5n - 1] = the state at the segment's end
   std::vector<StateBuf> ck(nseg + 1), sin(5 * (size_t)std::min<int64_t>(C, nsteps));
-  DevPtr lq, rq, lp, rp, G, ge, gp;
+  DevPtr slab, lq, rq, lp, rp, G, ge, gp;
   auto cleanup = [&]() {
-    for (auto& b : ck) free_state(b);
-    for (auto& b : sin) free_state(b);
-    for (DevPtr* d : {&lq, &rq, &lp, &rp, &G, &ge, &gp}) dfree(*d);
+    for (DevPtr* d : {&slab, &lq, &rq, &lp, &rp, &G, &ge, &gp}) dfree(*d);
   };
   auto fail_clean = [&](wadg_status st) {
     cleanup();
     return st;
   };
   wadg_status st = WADG_OK;
-  for (auto& b : ck) if ((st = alloc_state(ctx, b)) != WADG_OK) return fail_clean(st);
-  for (auto& b : sin) if ((st = alloc_state(ctx, b)) != WADG_OK) return fail_clean(st);
+  {
+    std::vector<StateBuf*> all;
+    for (auto& b : ck) all.push_back(&b);
+    for (auto& b : sin) all.push_back(&b);
+    if ((st = alloc_states(ctx, slab, all)) != WADG_OK) return fail_clean(st);
+  }
   const size_t qb = ctx->q[0].bytes, pb = ctx->p.bytes;
   cudaError_t ce = cudaSuccess;
   if (ce == cudaSuccess) ce = dalloc(lq, qb);
@@ -1811,6 +1794,9 @@ wadg_status adjoint_typed(wadg_ctx* ctx, int64_t nsteps, double dt, int C, doubl
   A.eps0_r = (Real)A.eps0;
   A.qslot = (const unsigned char*)ctx->qslot.p;
   A.nsl = 4 * sample_groups(ctx);
+  A.symadj = (const Real*)ctx->symadj.p; A.symtab = (const unsigned char*)ctx->symtab.p;
+  A.geox = (const Real*)ctx->geox.p; A.facex = (const Real*)ctx->facex.p;
+  A.err = (int*)ctx->errflag.p;
   for (int u = 0; u < 3; ++u) {
     A.sigma_max[u] = ctx->has_prof ? ctx->prof.sigma_max[u] : 0.0;
     A.p_sigma[u] = ctx->has_prof ? ctx->prof.p_sigma[u] : 0.0;
@@ -1855,11 +1841,13 @@ wadg_status adjoint_typed(wadg_ctx* ctx, int64_t nsteps, double dt, int C, doubl
         A.rk_a_r = (Real)A.rk_a;
         A.rk_b_r = (Real)A.rk_b;
         A.t = tn + kRkC.c[i] * dt;
-        CK(launch_adjoint_stage<Real>(ctx->N, A, nb, ctx->stream, ctx->qc));
+        CK(launch_adjoint_stage<Real>(ctx->N, A, nb, ctx->stream, ctx->qc, ctx->sym.G,
+                                      ctx->symcoef.data()));
       }
     }
   }
   CK(cudaStreamSynchronize(ctx->stream));
+  if ((st = check_err_flag(ctx)) != WADG_OK) return fail_clean(st);
   // final forward state back in place
   if ((st = load_state(ctx, ck[nseg])) != WADG_OK) return fail_clean(st);
   CK(cudaStreamSynchronize(ctx->stream));

@@ -477,6 +477,67 @@ template cudaError_t launch_pml_samples<double>(int, bool, int, int, const doubl
 template cudaError_t launch_pml_samples<float>(int, bool, int, int, const double*, const double*,
                                                const double*, float*, float*, bool, cudaStream_t);
 
+// Per-element tables of the symmetric stage (layouts: kernels.cuh), one thread
+// per face: the upwind flux's factors, evaluated in double from the stored
+// normals and impedances, and with face 0 the element's geometry.
+template <typename Real>
+__global__ void sym_geometry_kernel(int64_t K, const double* geo, const double* verts,
+                                    const Real* fnrm, const Real* mat, const int* nbr,
+                                    const unsigned char* code, Real* facex, Real* geox) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= 4 * K) return;
+  const int64_t e = i >> 2;
+  const double Zm = (double)mat[e * 3 + 2];
+  const double Zp = nbr[i] < 0 ? Zm : (double)mat[(int64_t)nbr[i] * 3 + 2];
+  const double w = (double)fnrm[i * 4 + 3] / (Zm + Zp);
+  Real* o = facex + i * 8;
+  for (int d = 0; d < 3; ++d) o[d] = fnrm[i * 4 + d];
+  o[3] = (Real)(Zp * w);
+  o[4] = (Real)w;
+  o[5] = (Real)(Zm * w);
+  o[6] = (Real)(Zm * Zp * w);
+  o[7] = (Real)code[i];
+  if (i & 3) return;
+  double X[3][3];   // column a: dx/dxi_a
+  const double* v = verts + e * 12;
+  for (int d = 0; d < 3; ++d) {
+    X[d][0] = 0.25 * (v[d] + v[3 + d] - v[6 + d] - v[9 + d]);
+    X[d][1] = 0.25 * (v[d] - v[3 + d] + v[6 + d] - v[9 + d]);
+    X[d][2] = 0.25 * (v[d] - v[3 + d] - v[6 + d] + v[9 + d]);
+  }
+  const double* g = geo + e * 9;   // grad r, s, t; grad xi_1 = -(grad s + grad t), ...
+  Real* x = geox + e * 12;
+  for (int k = 0; k < 9; ++k) {
+    const int a = k / 3, d = k % 3;
+    x[k] = sizeof(Real) == 8 ? (Real)X[a][d]
+                             : (Real)-(g[(a + 1) % 3 * 3 + d] + g[(a + 2) % 3 * 3 + d]);
+  }
+  x[9] = (Real)(1.0 / (X[0][0] * (X[1][1] * X[2][2] - X[1][2] * X[2][1]) -
+                       X[0][1] * (X[1][0] * X[2][2] - X[1][2] * X[2][0]) +
+                       X[0][2] * (X[1][0] * X[2][1] - X[1][1] * X[2][0])));
+  x[10] = mat[e * 3];
+  x[11] = mat[e * 3 + 1];
+}
+
+template <typename Real>
+cudaError_t launch_sym_geometry(int64_t K, const double* geo, const double* verts,
+                                const Real* fnrm, const Real* mat, const int* nbr,
+                                const unsigned char* code, Real* facex, Real* geox,
+                                cudaStream_t s) {
+  if (K == 0) return cudaSuccess;
+  sym_geometry_kernel<Real><<<(unsigned)((4 * K + 255) / 256), 256, 0, s>>>(
+      K, geo, verts, fnrm, mat, nbr, code, facex, geox);
+  return cudaGetLastError();
+}
+template cudaError_t launch_sym_geometry<double>(int64_t, const double*, const double*,
+                                                 const double*, const double*, const int*,
+                                                 const unsigned char*, double*, double*,
+                                                 cudaStream_t);
+template cudaError_t launch_sym_geometry<float>(int64_t, const double*, const double*,
+                                                const float*, const float*, const int*,
+                                                const unsigned char*, float*, float*,
+                                                cudaStream_t);
+
 template <typename Real>
 __global__ void check_finite_kernel(const Real* a, int64_t n, int* flag) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;

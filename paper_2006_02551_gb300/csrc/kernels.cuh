@@ -127,6 +127,13 @@ struct AdjParams {
   Real* G;                  // scratch [b][e][4 Nfp][6]
   double* grad_eps;         // [b][K] internal order
   double* grad_prof;        // [b][6]: d/dsigma_max[3], d/dp_sigma[3]
+  // FP32, symmetric kernels (sym_adjoint.cu)
+  const Real* symadj;       // transposed derivative blocks, LIFT^T blocks
+  const unsigned char* symtab;
+  const Real* geox;
+  const Real* facex;
+  int* err;                 // device error flag (bounded waits that gave up)
+  int tile;                 // elements per tile (set by the launcher)
   const double* geo;
   const Real* fnrm;         // [e][4][4]: unit outward normal, Fscale (as the forward stage)
   const Real* mat;
@@ -184,9 +191,18 @@ int sym_split(int N, int G, bool kappa, int64_t n);
 cudaError_t launch_probes(bool fp64, const ProbeParams& P, cudaStream_t s);
 template <typename Real>
 cudaError_t configure_adjoint_kernels(int N);
+// the reverse stage; FP32: G, coef the volume rule's symmetry and coefficients
+// (0: the dense PML kernel)
 template <typename Real>
-cudaError_t launch_adjoint_stage(int N, const AdjParams<Real>& P, int nb, cudaStream_t s,
-                                 int qc = 0);
+cudaError_t launch_adjoint_stage(int N, const AdjParams<Real>& P, int nb, cudaStream_t s, int qc,
+                                 int G, const float* coef);
+// FP32 with the operators in blocks: lift of every element, then the main part
+// of a class (G = 0 non-PML, 4 or 2 PML; coef as launch_sym's)
+bool sym_adjoint_built(int N, int G);
+cudaError_t configure_sym_adjoint(int N);
+cudaError_t launch_sym_lift(int N, const AdjParams<float>& P, int nb, cudaStream_t s);
+cudaError_t launch_sym_adjoint(int N, int G, const AdjParams<float>& P, const float* coef, int nb,
+                               cudaStream_t s);
 template <typename Real>
 cudaError_t launch_adjoint_probes(const Real* q, int64_t strideQ, int nprobe, int nb, int Np,
                                   const int* elem, const double* ell, Real* lam, cudaStream_t s);
@@ -201,6 +217,12 @@ cudaError_t configure_tc_rows(int N, bool bf16);
 cudaError_t launch_pml_tc_rows(int N, const StageParams<float>& P, int nb, cudaStream_t s,
                                bool bf16);
 cudaError_t launch_advance(double* t_dev, int64_t* step_dev, double dt, cudaStream_t s);
+// geox and facex of K elements from the other per-element tables
+template <typename Real>
+cudaError_t launch_sym_geometry(int64_t K, const double* geo, const double* verts,
+                                const Real* fnrm, const Real* mat, const int* nbr,
+                                const unsigned char* code, Real* facex, Real* geox,
+                                cudaStream_t s);
 // n sample places per element and axis at the reference points rq [n][3] (a
 // coordinate above 1: padding); groups: [group][3][4] blocks of sigma / eps0,
 // else [3][n] blocks of sigma

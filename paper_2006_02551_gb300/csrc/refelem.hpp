@@ -66,9 +66,16 @@ std::vector<double> sym_adapt(int N, const std::vector<double>& f);
 // Tables of the symmetric CUDA-core stage (layout: SymLayout): the
 // operators' blocks, and for each node m of face 0 and each element g_y of V4
 // the face-node index [Nfp][4] and the volume node [Nfp][4] of its image,
-// then the nodes of the node orbits and the node nearest the centroid.
+// then the nodes of the node orbits, the node nearest the centroid, and the (up
+// to three) face nodes at each node.
 void build_sym_tables(const RefOps& R, const SymRule& S, std::vector<double>& ops,
                       std::vector<unsigned char>& tabs);
+
+// The blocks of build_sym_tables transposed, in FP32: derivatives by output
+// character y and direction a (at d_off(y, a)), columns (value i of character y
+// xor a) of RP(y) rows; then LIFT^T, columns (value i of character x) of the
+// face-node orbits, padded to a multiple of four.
+std::vector<float> sym_transposed(int N, const std::vector<double>& ops);
 
 // the derivative and LIFT blocks of order N in FP32 (SymLayout order), built once
 const std::vector<float>& sym_constants(int N);

@@ -618,6 +618,18 @@ __device__ __forceinline__ void sym_add2(const float* coef, const float* v, cons
       }
     }
 }
+// the same for one row (constant-bank coefficients)
+template <int N, int G>
+__device__ __forceinline__ void sym_add1(const float* coef, const float* v, float* acc) {
+  using B = Blocks<N, G>;
+#pragma unroll
+  for (int o = 0; o < 4 / G; ++o)
+#pragma unroll
+    for (int x = 0; x < G; ++x)
+#pragma unroll
+      for (int j = 0; j < B::dim(x); ++j)
+        acc[B::off(x) + j] += coef[o * B::PO + B::poff(x) + j] * v[G * o + x];
+}
 // V4-adapted coefficients -> adapted sums: times the orbits' sizes
 template <typename Real, int N>
 __device__ __forceinline__ void sym_to_sums(Real* s) {

@@ -113,6 +113,15 @@ void tables(const RefOps& R, const SymRule& S, std::vector<double>& ops,
       }
     }
     tabs.push_back((unsigned char)nc);
+    for (int n = 0; n < Np; ++n) {   // the face nodes at each node (NF: none)
+      int k = 0;
+      for (int fm = 0; fm < NF && k < 3; ++fm)
+        if (R.Fmask[fm] == n) {
+          tabs.push_back((unsigned char)fm);
+          ++k;
+        }
+      for (; k < 3; ++k) tabs.push_back((unsigned char)NF);
+    }
   }
   if (S.G == 0) return;
   const auto TR = S.G == 4 ? T : node_sums_z2<N>();
@@ -203,6 +212,37 @@ SymRule detect_symmetry(const RefOps& R) {
     if ((int)S.slots.size() <= 4 * sym_groups(R.N, G)) return S;
   }
   return SymRule{};
+}
+
+namespace {
+template <int N>
+std::vector<float> transposed(const std::vector<double>& ops) {
+  using L = SymLayout<N>;
+  using B = Blocks<N, 4>;
+  constexpr int Nfp = L::Nfp, RM = (Nfp + 3) & ~3;
+  std::vector<float> t(L::oL + (size_t)B::Np * RM, 0.f);
+  for (int y = 0; y < 4; ++y)
+    for (int a = 1; a <= 3; ++a)
+      for (int i = 0; i < B::dim(y ^ a); ++i)
+        for (int j = 0; j < B::dim(y); ++j)
+          t[L::d_off(y, a) + i * L::RP(y) + j] =
+              (float)ops[L::d_off(y ^ a, a) + j * L::RP(y ^ a) + i];
+  for (int x = 0; x < 4; ++x)
+    for (int i = 0; i < B::dim(x); ++i)
+      for (int m = 0; m < Nfp; ++m)
+        t[L::oL + (size_t)(B::off(x) + i) * RM + m] = (float)ops[L::l_off(x) + m * L::RP(x) + i];
+  return t;
+}
+}  // namespace
+
+std::vector<float> sym_transposed(int N, const std::vector<double>& ops) {
+  switch (N) {
+    case 1: return transposed<1>(ops);
+    case 2: return transposed<2>(ops);
+    case 3: return transposed<3>(ops);
+    case 4: return transposed<4>(ops);
+    default: return transposed<5>(ops);
+  }
 }
 
 std::vector<double> sym_adapt(int N, const std::vector<double>& f) {
