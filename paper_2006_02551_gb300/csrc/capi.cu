@@ -565,6 +565,7 @@ wadg_status rebuild_typed(wadg_ctx* ctx) {
   CK(dalloc(ctx->code, code.size()));
   CK(cudaMemcpy(ctx->code.p, code.data(), code.size(), cudaMemcpyHostToDevice));
   if (!ctx->tc) {   // geometry, material and face factors of the symmetric stage
+    CK(cudaStreamSynchronize(cudaStreamLegacy));   // the copies above have landed
     CK(dalloc(ctx->facex, (size_t)K * 32 * sizeof(Real)));
     CK(dalloc(ctx->geox, (size_t)K * 12 * sizeof(Real)));
     CK((launch_sym_geometry<Real>(K, (const double*)ctx->geo.p, (const double*)ctx->verts.p,
@@ -882,10 +883,31 @@ wadg_status issue_stage_branches(wadg_ctx* ctx, int stage, double dt) {
   return WADG_OK;
 }
 
+// one stage of a step graph with both element classes in one launch; false in
+// *done where the class kernels are not of that kind or do not fit one wave
+template <typename Real>
+wadg_status issue_stage_both(wadg_ctx* ctx, int stage, double dt, bool* done) {
+  *done = false;
+  if (ctx->tc || !ctx->sym.G || ctx->scheme == WADG_PML_STORED) return WADG_OK;
+  const StageParams<Real> A = stage_params<Real>(ctx, stage, dt, 0.0, true, false);
+  const StageParams<Real> B = stage_params<Real>(ctx, stage, dt, 0.0, true, true);
+  CK(launch_sym_both<Real>(ctx->N, ctx->sym.G, ctx->kappa, A, B, ctx->symcoef.data(), ctx->nb,
+                           stage > 0, ctx->stream, done));
+  if (*done) ctx->cur ^= 1;
+  return WADG_OK;
+}
+
 wadg_status issue_step(wadg_ctx* ctx, double dt) {
   const bool branches = ctx->K1 > 0 && ctx->K0 > 0 && ctx->aux;
   for (int s = 0; s < 5; ++s) {
     wadg_status st;
+    bool done = false;
+    if (branches) {
+      st = ctx->rs == 8 ? issue_stage_both<double>(ctx, s, dt, &done)
+                        : issue_stage_both<float>(ctx, s, dt, &done);
+      if (st != WADG_OK) return st;
+      if (done) continue;
+    }
     if (branches)
       st = ctx->rs == 8 ? issue_stage_branches<double>(ctx, s, dt)
                         : issue_stage_branches<float>(ctx, s, dt);

@@ -184,6 +184,14 @@ cudaError_t configure_sym_kernels(int N);
 template <typename Real>
 cudaError_t launch_sym(int N, int G, bool kappa, const StageParams<Real>& P, const float* coef,
                        int nb, cudaStream_t s);
+// both classes of a stage (A: non-PML, B: PML) in one launch, where their tiles
+// fit one wave of blocks (*done: whether it was launched).  chained: the launch
+// follows the last stage's on the stream, and may set its tables up before that
+// one ends
+template <typename Real>
+cudaError_t launch_sym_both(int N, int G, bool kappa, const StageParams<Real>& A,
+                            const StageParams<Real>& B, const float* coef, int nb, bool chained,
+                            cudaStream_t s, bool* done);
 // threads that share a row's point groups in a class of n elements (times
 // excitations); the same for every launch of the class, whatever its tiles
 template <typename Real>

@@ -735,7 +735,12 @@ __device__ __forceinline__ void sym_body(const StageParams<Real>& P, const SymCo
     copy_in(src, len, dst, 2, mf);
   };
   uint32_t phase = 0;   // tiles done: the barriers' parities
-  bool failed = false, ahead = false;   // ahead: this tile's faces are on their way
+  bool failed = false, ahead = !dyn && bid < ntiles;   // ahead: this tile's faces are on their way
+  if (ahead && tid == 0) faces_in(bid, 0);
+  // in a chained launch: the next stage may start its set-up, and this one's
+  // reads of the state wait for the last stage's writes (no-ops otherwise)
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   claim();
   for (int tile = next_tile(-1); tile < ntiles; tile = next_tile(tile), ++phase) {
     claim();
