@@ -656,7 +656,7 @@ def main():
         # tensor-core contractions: the stage is bound by HBM traffic
         traffic = (tc_pml_traffic(K1 * w.n_batch, N, args.precision)
                    if dom == "pml" and rows else None)
-        kname = "tc_rows_kernel" if (rows and dom == "pml") else "tc_stage_kernel"
+        kname = "tc_stage_kernel" if (dom == "pml" and not rows) else "tc_rows_kernel"
         roofline = {"bound": "hbm", "achieved": achieved_gbs, "peak": hbm, "unit": "GB/s",
                     "frac": achieved_gbs / hbm, "traffic": traffic,
                     "traffic_note": "ncu DRAM bytes per PML element of the 24^3 case (mean "
@@ -671,7 +671,7 @@ def main():
         peak_note = (f"measured {'FP64' if args.precision == 'fp64' else 'FP32'} FMA "
                      f"throughput (wadg_fma_peak: register FMA chains on every SM)")
         roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                    "frac": achieved / peak, "traffic": None, "kernel": f"stage_kernel<{dom}>",
+                    "frac": achieved / peak, "traffic": None, "kernel": f"sym_stage_kernel<{dom}>",
                     "peak_source": peak_note,
                     "hbm": {"achieved_gbs": achieved_gbs, "peak_gbs": hbm,
                             "frac": achieved_gbs / hbm}}

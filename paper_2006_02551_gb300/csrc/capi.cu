@@ -799,8 +799,8 @@ cudaError_t launch_pml_class(wadg_ctx* ctx, const StageParams<Real>& P, cudaStre
   if constexpr (std::is_same<Real, float>::value) {
     if (ctx->tc) {
       // compact volume rules: the row-owned kernel; (N+1)^3 rules: the other
-      if (ctx->qc == 1) return launch_pml_tc_rows(ctx->N, P, ctx->nb, s, ctx->bf16);
-      return launch_stage_tc(ctx->N, true, P, ctx->nb, s, ctx->bf16, ctx->qc);
+      if (ctx->qc == 1) return launch_tc_rows(ctx->N, true, P, ctx->nb, s, ctx->bf16);
+      return launch_pml_tc(ctx->N, P, ctx->nb, s, ctx->bf16);
     }
   }
   // CUDA cores: the symmetric stage, or for a rule without symmetry the dense one
@@ -817,7 +817,7 @@ cudaError_t launch_pml_class(wadg_ctx* ctx, const StageParams<Real>& P) {
 template <typename Real>
 cudaError_t launch_std_class(wadg_ctx* ctx, const StageParams<Real>& P, cudaStream_t s) {
   if constexpr (std::is_same<Real, float>::value)
-    if (ctx->tc) return launch_stage_tc(ctx->N, false, P, ctx->nb, s, ctx->bf16, ctx->qc);
+    if (ctx->tc) return launch_tc_rows(ctx->N, false, P, ctx->nb, s, ctx->bf16);
   return launch_sym<Real>(ctx->N, 0, false, P, nullptr, ctx->nb, s);
 }
 
@@ -840,7 +840,7 @@ template <typename Real>
 wadg_status issue_stage(wadg_ctx* ctx, int stage, double dt, double t, bool use_tdev) {
   if (ctx->tc) {
     StageParams<float> A = stage_params<float>(ctx, stage, dt, t, use_tdev, false);
-    CK(launch_stage_tc(ctx->N, false, A, ctx->nb, ctx->stream, ctx->bf16, ctx->qc));
+    CK(launch_tc_rows(ctx->N, false, A, ctx->nb, ctx->stream, ctx->bf16));
     if (ctx->K1 > 0) {
       StageParams<float> B = stage_params<float>(ctx, stage, dt, t, use_tdev, true);
       CK(launch_pml_class<float>(ctx, B));
@@ -870,7 +870,7 @@ wadg_status issue_stage_branches(wadg_ctx* ctx, int stage, double dt) {
     StageParams<float> B = stage_params<float>(ctx, stage, dt, 0.0, true, true);
     CK(launch_pml_class<float>(ctx, B));
     StageParams<float> A = stage_params<float>(ctx, stage, dt, 0.0, true, false);
-    CK(launch_stage_tc(ctx->N, false, A, ctx->nb, ctx->aux, ctx->bf16, ctx->qc));
+    CK(launch_tc_rows(ctx->N, false, A, ctx->nb, ctx->aux, ctx->bf16));
   } else {
     StageParams<Real> B = stage_params<Real>(ctx, stage, dt, 0.0, true, true);
     CK(launch_pml_class<Real>(ctx, B));
@@ -2060,7 +2060,7 @@ wadg_status noalloc_stage(wadg_ctx* ctx, int stage, double dt, const double* tde
   if (ctx->tc) {
     StageParams<float> A = stage_params<float>(ctx, stage, dt, 0.0, false, false);
     A.t_dev = tdev;
-    CK(launch_stage_tc(ctx->N, false, A, ctx->nb, ctx->stream, ctx->bf16, ctx->qc));
+    CK(launch_tc_rows(ctx->N, false, A, ctx->nb, ctx->stream, ctx->bf16));
     if (ctx->K1 > 0) {
       StageParams<float> B = stage_params<float>(ctx, stage, dt, 0.0, false, true);
       B.t_dev = tdev;

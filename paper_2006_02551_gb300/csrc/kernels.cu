@@ -449,13 +449,12 @@ __global__ void pml_samples_kernel(int n, bool groups, int K1, int K0, const dou
   const double t = element_constant ? -0.5 : rq[q * 3 + 2];
   const double l0 = -0.5 * (1 + r + s + t), l1 = 0.5 * (1 + r), l2 = 0.5 * (1 + s),
                l3 = 0.5 * (1 + t);
-  const double scale = groups ? 1.0 / prof[15] : 1.0;
   for (int u = 0; u < 3; ++u) {
     const double x = l0 * v[u] + l1 * v[3 + u] + l2 * v[6 + u] + l3 * v[9 + u];
     const double d = (fabs(x) - prof[u]) / prof[3 + u];
     double g = 0.0;
     if (d > 0) g = pow(d, prof[9 + u]);
-    sig[at(u)] = (Real)(prof[6 + u] * g * scale);
+    sig[at(u)] = (Real)(prof[6 + u] * g * (1.0 / prof[15]));
     if (kap) kap[at(u)] = (Real)(1.0 + (prof[12 + u] - 1.0) * g);
   }
 }

@@ -24,7 +24,7 @@
 //            CUDA-core contexts: sigma_u/eps0 and kappa_u as
 //            [e'][group][3][4], the nodes in groups of four in the order of
 //            the rule's symmetry (SymRule; its own order without one);
-//            tensor-core contexts: sigma_u as [e'][3][Nq]
+//            tensor-core contexts: sigma_u/eps0 as [e'][3][Nq]
 //            stored[e'][3][3][Np][NpP]  stored-matrix scheme: per axis u the
 //            operators M_k^-1 M_k^{b_u}, M_k^-1 M_k^{c_u}, M_k^-1 M_k^{d_u},
 //            transposed (column j of the operator is row j here)
@@ -218,12 +218,12 @@ cudaError_t launch_adjoint_probes(const Real* q, int64_t strideQ, int nprobe, in
 // tc_supported: whether a tensor-core stage exists for (N, bf16, qc)
 bool tc_supported(int N, bool kappa, bool bf16, int qc = 0);
 cudaError_t configure_tc_kernels(int N, bool bf16);
-cudaError_t launch_stage_tc(int N, bool pml, const StageParams<float>& P, int nb, cudaStream_t s,
-                            bool bf16, int qc = 0);
-// row-owned tensor-core PML stage kernels (compact volume rules)
+cudaError_t launch_pml_tc(int N, const StageParams<float>& P, int nb, cudaStream_t s, bool bf16);
+// row-owned tensor-core stage kernels: the non-PML class, and the PML class
+// with compact volume rules
 cudaError_t configure_tc_rows(int N, bool bf16);
-cudaError_t launch_pml_tc_rows(int N, const StageParams<float>& P, int nb, cudaStream_t s,
-                               bool bf16);
+cudaError_t launch_tc_rows(int N, bool pml, const StageParams<float>& P, int nb, cudaStream_t s,
+                           bool bf16);
 cudaError_t launch_advance(double* t_dev, int64_t* step_dev, double dt, cudaStream_t s);
 // geox and facex of K elements from the other per-element tables
 template <typename Real>
@@ -233,7 +233,7 @@ cudaError_t launch_sym_geometry(int64_t K, const double* geo, const double* vert
                                 cudaStream_t s);
 // n sample places per element and axis at the reference points rq [n][3] (a
 // coordinate above 1: padding); groups: [group][3][4] blocks of sigma / eps0,
-// else [3][n] blocks of sigma
+// else [3][n] blocks of it
 template <typename Real>
 cudaError_t launch_pml_samples(int n, bool groups, int K1, int K0, const double* verts,
                                const double* rq, const double* prof /*16*/, Real* sig, Real* kap,

@@ -31,24 +31,22 @@
 namespace wadg {
 namespace tc {
 
-// Shared-memory plan of one tile (all offsets in bytes).  QC: quadrature
-// class of the volume rule (quad_capacity).
-template <int N, bool PML, bool BF = false, int QC = 0>
+// Shared-memory plan of one tile (all offsets in bytes).  
+template <int N, bool BF>
 struct Plan {
   using O = OpT<BF>;
   static constexpr int Np = (N + 1) * (N + 2) * (N + 3) / 6;
   static constexpr int Nfp = (N + 1) * (N + 2) / 2;
   static constexpr int NF = 4 * Nfp;
-  static constexpr int Nq = quad_capacity(N, QC);
+  static constexpr int Nq = quad_capacity(N, 0);   // (N+1)^3
   __host__ __device__ static constexpr int rupK(int x) { return (x + O::KS - 1) / O::KS * O::KS; }
   static constexpr int NpK = rupK(Np), NFK = rupK(NF), NqK = rupK(Nq);
-  // elements per tile: 8; 4 for BF16 PML tiles, whose smaller operands then
-  // let two blocks share an SM (N <= 4) or fit at all (N = 5), and for TF32
-  // PML tiles at N = 5 (compact rule only)
-  static constexpr bool PAIR = PML && BF && N <= 4;
-  static constexpr int T = PML && (BF || N == 5) ? 4 : 8;
-  // one block per SM with 16 compute warps (TF32 PML; every N = 5 tile)
-  static constexpr bool ONE = PML ? !PAIR : N == 5;
+  // elements per tile: 8; 4 for BF16 tiles, whose smaller operands then let
+  // two blocks share an SM (N <= 4) or fit at all (N = 5)
+  static constexpr bool PAIR = BF && N <= 4;
+  static constexpr int T = BF ? 4 : 8;
+  // one block per SM with 16 compute warps (TF32, and N = 5)
+  static constexpr bool ONE = !PAIR;
   static constexpr int NV = rup16(6 * T);            // columns of E,H products
   static constexpr int NQ = rup16(12 * T);           // columns of 12-component products
   static constexpr int G_p = NpK / 8;                // 8-row groups of an Np-row operator
@@ -64,7 +62,7 @@ struct Plan {
   }
   // A operands
   static constexpr uint32_t oPq = 0;
-  static constexpr uint32_t oL = PML ? oPq + G_p * SBO_Q : 0;
+  static constexpr uint32_t oL = oPq + G_p * SBO_Q;
   // Dr, Ds, Dt stacked as one operator of 3 Np rows (row d Np + i), read as
   // VT products of up to 128 rows: DPT derivatives per product (N <= 4: all
   // three in one; N = 5: [Dr; Ds], then Dt)
@@ -78,18 +76,17 @@ struct Plan {
   // buffers that follow it
   static constexpr int VQT = (Nq + 127) / 128;
   // B operands
-  static constexpr uint32_t oBF = PML ? oVq + (rup8(Nq) / 8) * SBO_V : oVq;
-  static constexpr int ROWS_F = PML ? NQ : NV;        // E,H (+ P) rows
+  static constexpr uint32_t oBF = oVq + (rup8(Nq) / 8) * SBO_V;
+  static constexpr int ROWS_F = NQ;                   // E,H and P rows
   static constexpr uint32_t oBFL = oBF + (ROWS_F / 8) * SBB_V;
   static constexpr uint32_t oBTZ = oBFL + (NV / 8) * SBB_L;
   // the (t, z) operand buffer later holds the P_q columns copied out of
   // TMEM ([T][12][Np] floats), which can be the larger of the two
   static constexpr uint32_t BTZ_BYTES = (NQ / 8) * SBB_Q;
   static constexpr uint32_t DP_BYTES = T * 12 * Np * 4;
-  static constexpr uint32_t oRS =
-      PML ? oBTZ + (BTZ_BYTES > DP_BYTES ? BTZ_BYTES : DP_BYTES) : oBTZ;
+  static constexpr uint32_t oRS = oBTZ + (BTZ_BYTES > DP_BYTES ? BTZ_BYTES : DP_BYTES);
   static constexpr int NpP = (Np + 3) & ~3;
-  static constexpr uint32_t oGeo = oRS + (PML ? T * 6 * NpP * 4 : 0);
+  static constexpr uint32_t oGeo = oRS + T * 6 * NpP * 4;
   static constexpr int TS = T * 6 * Np;               // floats of one staged field block
   // a staged block is the 16-byte-aligned cover of the element block: up to
   // 8 bytes more at each end
@@ -100,7 +97,7 @@ struct Plan {
   static constexpr uint32_t GFN = ((T * 64 + 15) & ~15) + 16;
   static constexpr uint32_t GMET = ((T * 72 + 15) & ~15) + 16;
   static constexpr uint32_t GMAT = ((T * 12 + 15) & ~15) + 16;
-  static constexpr uint32_t oSFN = (PML ? 4 : 2) * TSB;   // offsets within a set
+  static constexpr uint32_t oSFN = 4 * TSB;   // offsets within a set
   static constexpr uint32_t oSMET = oSFN + GFN;
   static constexpr uint32_t oSMAT = oSMET + GMET;
   static constexpr uint32_t SET = oSMAT + GMAT;
@@ -123,23 +120,23 @@ struct Plan {
   static constexpr uint32_t DV_BYTES = T * DVE * 4;
   // (BF16 operand buffers are too small for the volume/LIFT dump: it gets its
   // own region)
-  static constexpr bool DV_ALIAS = PML && !BF;
+  static constexpr bool DV_ALIAS = !BF;
   static constexpr uint32_t oDV = DV_ALIAS ? oBF : oMisc + MISC_BYTES;
   static constexpr uint32_t oDP = oBTZ;
   static_assert(!DV_ALIAS || oDV + DV_BYTES <= oBTZ, "volume/LIFT dump");
-  static_assert(!PML || oDP + DP_BYTES <= oRS, "P_q dump");
+  static_assert(oDP + DP_BYTES <= oRS, "P_q dump");
   static constexpr uint32_t bytes_used = DV_ALIAS ? oMisc + MISC_BYTES : oDV + DV_BYTES;
   // residency follows the tensor-memory budget of 512 columns per SM: one
   // TF32 PML block (512 columns) per SM, enforced by the shared-memory request
-  // so that no block waits in tcgen05.alloc; BF16 PML blocks (256 columns)
-  // and non-PML blocks (128 columns) two per SM (shared memory, registers)
+  // so that no block waits in tcgen05.alloc; BF16 blocks (256 columns) two
+  // per SM (shared memory, registers)
   static constexpr uint32_t min_bytes = ONE ? 116 * 1024 : 100 * 1024;
   static constexpr uint32_t bytes = bytes_used < min_bytes ? min_bytes : bytes_used;
   // TMEM column bases: derivative products (lanes d Np + i of product v at
   // cV + v NV), LIFT, V_q products (cVq + t NQ), P_q
   static constexpr uint32_t cV = 0, cL = VT * NV;
   static constexpr uint32_t cVq = cL + NV, cPq = cVq + VQT * NQ;
-  static constexpr uint32_t COLS = PML ? cPq + NQ : cL + NV;
+  static constexpr uint32_t COLS = cPq + NQ;
   static constexpr uint32_t TMEM_COLS = COLS <= 128 ? 128 : (COLS <= 256 ? 256 : 512);
   static_assert(COLS <= 512, "TMEM columns");
   static_assert(!PAIR || (bytes <= 113 * 1024 && TMEM_COLS <= 256), "two BF16 PML blocks per SM");
@@ -148,10 +145,10 @@ struct Plan {
   static_assert(VT <= 2 && VQT <= 2, "at most two products per operator");
   static_assert(Np <= 64, "node rows");
   // every A operand read (128 rows from its start) stays inside the block
-  static_assert(oPq + 16 * SBO_Q <= bytes || !PML, "P_q span");
+  static_assert(oPq + 16 * SBO_Q <= bytes, "P_q span");
   static_assert(oL + 16 * SBO_L <= bytes, "LIFT span");
   static_assert(oVol + ((VT - 1) * DPT * Np / 8 + 16) * SBO_V <= bytes, "volume operator span");
-  static_assert(!PML || oVq + 16 * VQT * SBO_V <= bytes, "V_q span");
+  static_assert(oVq + 16 * VQT * SBO_V <= bytes, "V_q span");
   static_assert(VQT == 1 || Nq % 8 == 0, "second V_q product starts on a row group");
   static_assert(bytes <= 227 * 1024, "shared memory");
 };
@@ -168,9 +165,9 @@ struct Plan {
 // launch allocation to the compute warps (setmaxnreg), which removes their
 // spills (the launch holds every thread to the share of 5 or 6 warps per
 // scheduler).
-template <int N, bool PML, bool BF, int QC = 0>
+template <int N, bool BF>
 struct TcWarps {
-  static constexpr bool ONE = Plan<N, PML, BF, QC>::ONE;   // one block per SM
+  static constexpr bool ONE = Plan<N, BF>::ONE;   // one block per SM
   static constexpr int compute = ONE ? 16 : 8;
   static constexpr int issue = 4;
   static constexpr int threads = 32 * (compute + issue);
@@ -187,12 +184,12 @@ struct TcWarps {
                 "register split within the launch allocation");
 };
 
-template <int N, bool PML, bool BF, int QC>
-__global__ void __launch_bounds__(TcWarps<N, PML, BF, QC>::threads,
-                                  TcWarps<N, PML, BF, QC>::ONE ? 1 : 2)
+template <int N, bool BF>
+__global__ void __launch_bounds__(TcWarps<N, BF>::threads,
+                                  TcWarps<N, BF>::ONE ? 1 : 2)
     tc_stage_kernel(const StageParams<float> P) {
-  using PL = Plan<N, PML, BF, QC>;
-  using TW = TcWarps<N, PML, BF, QC>;
+  using PL = Plan<N, BF>;
+  using TW = TcWarps<N, BF>;
   constexpr int NW = TW::compute;
   constexpr int kTcThreads = 32 * NW;          // compute threads
   constexpr int kAll = TW::threads;
@@ -240,15 +237,13 @@ __global__ void __launch_bounds__(TcWarps<N, PML, BF, QC>::threads,
       const int i = idx / NF, f = idx - i * NF;
       put_op<BF>(smem + PL::oL + PL::ofs(i, f, PL::SBO_L, PL::LA), gL[idx]);
     }
-    if (PML) {
-      for (int idx = tid; idx < Nq * Np; idx += kAll) {
-        const int q = idx / Np, j = idx - q * Np;
-        put_op<BF>(smem + PL::oVq + PL::ofs(q, j, PL::SBO_V, PL::LA), gVq[idx]);
-      }
-      for (int idx = tid; idx < Np * Nq; idx += kAll) {
-        const int i = idx / Nq, q = idx - i * Nq;
-        put_op<BF>(smem + PL::oPq + PL::ofs(i, q, PL::SBO_Q, PL::LA), gPq[idx]);
-      }
+    for (int idx = tid; idx < Nq * Np; idx += kAll) {
+      const int q = idx / Np, j = idx - q * Np;
+      put_op<BF>(smem + PL::oVq + PL::ofs(q, j, PL::SBO_V, PL::LA), gVq[idx]);
+    }
+    for (int idx = tid; idx < Np * Nq; idx += kAll) {
+      const int i = idx / Nq, q = idx - i * Nq;
+      put_op<BF>(smem + PL::oPq + PL::ofs(i, q, PL::SBO_Q, PL::LA), gPq[idx]);
     }
   }
   for (int s = tid; s < min(P.nsrc, kSrcCache); s += kAll) {
@@ -300,7 +295,7 @@ __global__ void __launch_bounds__(TcWarps<N, PML, BF, QC>::threads,
   // set `set`: a block is copied as its 16-byte-aligned cover, so its first
   // value sits (address mod 16) bytes into the buffer.  (The library's
   // buffers end with spare bytes, so a cover never leaves its allocation.)
-  constexpr int NBLK = PML ? 4 : 2;
+  constexpr int NBLK = 4;
   auto tile_blocks = [&](int tile, const float* (&g)[4]) {
     const int b = tile / tiles_per_batch;
     const int t0 = (tile - b * tiles_per_batch) * T;
@@ -308,8 +303,8 @@ __global__ void __launch_bounds__(TcWarps<N, PML, BF, QC>::threads,
     const int64_t op = (int64_t)b * P.strideP + (int64_t)(P.e_begin + t0 - P.K0) * 6 * Np;
     g[0] = P.qin + oq;
     g[1] = P.resq + oq;
-    g[2] = PML ? P.p + op : nullptr;
-    g[3] = PML ? P.resp + op : nullptr;
+    g[2] = P.p + op;
+    g[3] = P.resp + op;
   };
   auto staged = [&](int set, int a, const float* g) {
     return reinterpret_cast<float*>(smem + PL::oST + set * PL::SET + a * PL::TSB +
@@ -413,14 +408,13 @@ __global__ void __launch_bounds__(TcWarps<N, PML, BF, QC>::threads,
     }
   };
   constexpr int VQT = PL::VQT;
-  auto load_sig = [&](int tile, float (&sgv)[PML ? EH : 1][VQT][3]) {
-    if (!PML) return;
+  auto load_sig = [&](int tile, float (&sgv)[EH][VQT][3]) {
     const int b = tile / tiles_per_batch;
     const int t0 = (tile - b * tiles_per_batch) * T;
     const int ne = min(T, P.n_elem - t0);
     const int ep0 = P.e_begin + t0 - P.K0;
 #pragma unroll
-    for (int k = 0; k < (PML ? EH : 1); ++k) {
+    for (int k = 0; k < EH; ++k) {
       const int e = grp + NGRP * k;
 #pragma unroll
       for (int t = 0; t < VQT; ++t) {
@@ -471,14 +465,13 @@ __global__ void __launch_bounds__(TcWarps<N, PML, BF, QC>::threads,
       int mit = 0;
       for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++mit) {
         if (!wait_ready(0)) { mfail = true; break; }
-        if (PML) {   // V_q first: the quadrature epilogue waits for it alone
-          for (int t = 0; t < PL::VQT; ++t)   // rows 128 t .. 128 t + 127
-            for (int k = 0; k < NpK / KS; ++k)
-              mma(tmem + PL::cVq + t * PL::NQ,
-                  make_desc(sbase + PL::oVq + 16 * t * PL::SBO_V + 256 * k, 128, PL::SBO_V),
-                  make_desc(sbase + PL::oBF + 2 * PL::LB * k, PL::LB, PL::SBB_V), idQ, k > 0);
-          mma_commit(saddr(mbar + 0));
-        }
+        // V_q first: the quadrature epilogue waits for it alone
+        for (int t = 0; t < PL::VQT; ++t)   // rows 128 t .. 128 t + 127
+          for (int k = 0; k < NpK / KS; ++k)
+            mma(tmem + PL::cVq + t * PL::NQ,
+                make_desc(sbase + PL::oVq + 16 * t * PL::SBO_V + 256 * k, 128, PL::SBO_V),
+                make_desc(sbase + PL::oBF + 2 * PL::LB * k, PL::LB, PL::SBB_V), idQ, k > 0);
+        mma_commit(saddr(mbar + 0));
         for (int v = 0; v < PL::VT; ++v)   // derivatives DPT v .. DPT v + DPT - 1
           for (int k = 0; k < NpK / KS; ++k)
             mma(tmem + PL::cV + v * PL::NV,
@@ -497,13 +490,11 @@ __global__ void __launch_bounds__(TcWarps<N, PML, BF, QC>::threads,
                    make_desc(sbase + PL::oBFL + 2 * PL::LB * k, PL::LB, PL::SBB_L), idV, k > 0);
         if (!withhold) mma_commit(saddr(mbar + 1));
         withhold = false;
-        if (PML) {
-          if (!wait_ready(2)) { mfail = true; break; }
-          for (int k = 0; k < NqK / KS; ++k)
-            mma(tmem + PL::cPq, make_desc(sbase + PL::oPq + 256 * k, 128, PL::SBO_Q),
-                     make_desc(sbase + PL::oBTZ + 2 * PL::LB * k, PL::LB, PL::SBB_Q), idQ, k > 0);
-          mma_commit(saddr(mbar + 2));
-        }
+        if (!wait_ready(2)) { mfail = true; break; }
+        for (int k = 0; k < NqK / KS; ++k)
+          mma(tmem + PL::cPq, make_desc(sbase + PL::oPq + 256 * k, 128, PL::SBO_Q),
+                   make_desc(sbase + PL::oBTZ + 2 * PL::LB * k, PL::LB, PL::SBB_Q), idQ, k > 0);
+        mma_commit(saddr(mbar + 2));
       }
       // the staging copies this thread issued land before the memory is released
       for (int s2 = 0; s2 < 2; ++s2)
@@ -522,7 +513,7 @@ __global__ void __launch_bounds__(TcWarps<N, PML, BF, QC>::threads,
   asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(TW::compute_regs));
   float Ep[FT][3], Hp[FT][3], ZPv[FT];
   int nbv[FT], codev[FT];
-  float sgv[PML ? EH : 1][VQT][3];
+  float sgv[EH][VQT][3];
   if ((int)blockIdx.x < ntiles) {
     load_nbr_idx(blockIdx.x, nbv, codev);
     load_nbr_val(blockIdx.x, nbv, codev, Ep, Hp, ZPv);
@@ -537,8 +528,8 @@ __global__ void __launch_bounds__(TcWarps<N, PML, BF, QC>::threads,
     tile_blocks(tile, gblk);
     float* SQ = staged(set, 0, gblk[0]);
     float* SR = staged(set, 1, gblk[1]);
-    float* SP = PML ? staged(set, 2, gblk[2]) : nullptr;
-    float* SRP = PML ? staged(set, 3, gblk[3]) : nullptr;
+    float* SP = staged(set, 2, gblk[2]);
+    float* SRP = staged(set, 3, gblk[3]);
     const int b = tile / tiles_per_batch;
     const int t0 = (tile - b * tiles_per_batch) * T;
     const int ne = min(T, P.n_elem - t0);
@@ -588,9 +579,9 @@ __global__ void __launch_bounds__(TcWarps<N, PML, BF, QC>::threads,
       for (int it2 = 0; it2 < NIT; ++it2) {
         const int task = tid + it2 * kTcThreads;
         const int row = task / G4, g = task - row * G4;
-        const int rr = PML && row >= 6 * T ? row - 6 * T : row;
+        const int rr = row >= 6 * T ? row - 6 * T : row;
         const bool live = task < NTASK && rr < ne * 6;
-        const float* src = (PML && row >= 6 * T ? SP : SQ) + rr * Np + CW * g;
+        const float* src = (row >= 6 * T ? SP : SQ) + rr * Np + CW * g;
 #pragma unroll
         for (int h = 0; h < CW; ++h) x[it2][h] = live && CW * g + h < Np ? src[h] : 0.f;
       }
@@ -598,7 +589,7 @@ __global__ void __launch_bounds__(TcWarps<N, PML, BF, QC>::threads,
       for (int it2 = 0; it2 < NIT; ++it2) {
         const int task = tid + it2 * kTcThreads;
         const int row = task / G4, g = task - row * G4;
-        const int rr = PML && row >= 6 * T ? row - 6 * T : row;
+        const int rr = row >= 6 * T ? row - 6 * T : row;
         if (task >= NTASK || rr >= ne * 6) continue;
         unsigned char* dst = smem + PL::oBF + PL::ofs(row, CW * g, PL::SBB_V, PL::LB);
         if constexpr (BF) {
@@ -669,66 +660,62 @@ __global__ void __launch_bounds__(TcWarps<N, PML, BF, QC>::threads,
     if (tid < ne * 9) geoM[(tid / 9) * 12 + tid % 9] = (float)met_s[tid];
     if (tid < ne * 2) geoM[(tid >> 1) * 12 + 9 + (tid & 1)] = mat_s[(tid >> 1) * 3 + (tid & 1)];
 
-    if (PML) {
-      if (!wait_bar(0)) { failed = true; break; }   // V_q product
-      // ---- epilogue A1: eq. 9 at the quadrature points -> B of P_q
-      {
-        const float ie0 = 1.f / (float)P.eps0;
+    if (!wait_bar(0)) { failed = true; break; }   // V_q product
+    // ---- epilogue A1: eq. 9 at the quadrature points -> B of P_q
+    {
 #pragma unroll
-        for (int t = 0; t < VQT; ++t) {       // V_q product t: points 128 t + lane row
-        const uint32_t cq = PL::cVq + t * PL::NQ;
-        // this lane's columns of the group's elements grp + NGRP k (warp-uniform);
-        // with two per group both loads are in flight before one wait
-        float vv[EH][12];
-        if constexpr (EH == 2 && 2 * NGRP == T) {
-          float w[24];
-          tld_6x2x2(tmem + lane_base + cq + grp * 6, tmem + lane_base + cq + 6 * T + grp * 6,
-                    tmem + lane_base + cq + (grp + NGRP) * 6,
-                    tmem + lane_base + cq + 6 * T + (grp + NGRP) * 6, w);
+      for (int t = 0; t < VQT; ++t) {       // V_q product t: points 128 t + lane row
+      const uint32_t cq = PL::cVq + t * PL::NQ;
+      // this lane's columns of the group's elements grp + NGRP k (warp-uniform);
+      // with two per group both loads are in flight before one wait
+      float vv[EH][12];
+      if constexpr (EH == 2 && 2 * NGRP == T) {
+        float w[24];
+        tld_6x2x2(tmem + lane_base + cq + grp * 6, tmem + lane_base + cq + 6 * T + grp * 6,
+                  tmem + lane_base + cq + (grp + NGRP) * 6,
+                  tmem + lane_base + cq + 6 * T + (grp + NGRP) * 6, w);
 #pragma unroll
-          for (int i = 0; i < 12; ++i) { vv[0][i] = w[i]; vv[1][i] = w[12 + i]; }
-        } else {
-#pragma unroll
-          for (int k = 0; k < EH; ++k) {
-            const int e = grp + NGRP * k;
-            if (e < T)
-              tld_6x2(tmem + lane_base + cq + e * 6, tmem + lane_base + cq + 6 * T + e * 6, vv[k]);
-          }
-        }
+        for (int i = 0; i < 12; ++i) { vv[0][i] = w[i]; vv[1][i] = w[12 + i]; }
+      } else {
 #pragma unroll
         for (int k = 0; k < EH; ++k) {
-          const int q = 128 * t + quad * 32 + lane;   // quadrature point of this lane
           const int e = grp + NGRP * k;
-          if (e >= T) break;
-          const float* v = vv[k];
-          if (e >= ne || q >= NqK) continue;
-          // sigma_u / eps0 at this point
-          const float sg[3] = {sgv[k][t][0] * ie0, sgv[k][t][1] * ie0, sgv[k][t][2] * ie0};
-          float o[12];
-#pragma unroll
-          for (int u = 0; u < 3; ++u) {
-            const float su = sg[u], sv = sg[(u + 1) % 3], sw = sg[(u + 2) % 3];
-            // eq. 9 with kappa = 1 in terms of s = sigma / eps0: a = 1,
-            // b = sv + sw - su, c = sv sw - b su
-            const float bc = sv + sw - su;
-            const float cc = sv * sw - bc * su;
-            const float dd = su;
-            o[u] = bc * v[u] + cc * v[6 + u];
-            o[3 + u] = bc * v[3 + u] + cc * v[9 + u];
-            o[6 + u] = v[u] - dd * v[6 + u];
-            o[9 + u] = v[3 + u] - dd * v[9 + u];
-          }
-#pragma unroll
-          for (int c = 0; c < 6; ++c) {
-            put_op<BF>(smem + PL::oBTZ + PL::ofs(e * 6 + c, q, PL::SBB_Q, PL::LB), o[c]);
-            put_op<BF>(smem + PL::oBTZ + PL::ofs(6 * T + e * 6 + c, q, PL::SBB_Q, PL::LB), o[6 + c]);
-          }
+          if (e < T)
+            tld_6x2(tmem + lane_base + cq + e * 6, tmem + lane_base + cq + 6 * T + e * 6, vv[k]);
         }
-        }   // t
       }
-      if (next < ntiles) load_sig(next, sgv);
-      signal_ready(5);   // P_q operand; the product overlaps the epilogue below
+#pragma unroll
+      for (int k = 0; k < EH; ++k) {
+        const int q = 128 * t + quad * 32 + lane;   // quadrature point of this lane
+        const int e = grp + NGRP * k;
+        if (e >= T) break;
+        const float* v = vv[k];
+        if (e >= ne || q >= NqK) continue;
+        const float* sg = sgv[k][t];   // sigma_u / eps0 at this point
+        float o[12];
+#pragma unroll
+        for (int u = 0; u < 3; ++u) {
+          const float su = sg[u], sv = sg[(u + 1) % 3], sw = sg[(u + 2) % 3];
+          // eq. 9 with kappa = 1 in terms of s = sigma / eps0: a = 1,
+          // b = sv + sw - su, c = sv sw - b su
+          const float bc = sv + sw - su;
+          const float cc = sv * sw - bc * su;
+          const float dd = su;
+          o[u] = bc * v[u] + cc * v[6 + u];
+          o[3 + u] = bc * v[3 + u] + cc * v[9 + u];
+          o[6 + u] = v[u] - dd * v[6 + u];
+          o[9 + u] = v[3 + u] - dd * v[9 + u];
+        }
+#pragma unroll
+        for (int c = 0; c < 6; ++c) {
+          put_op<BF>(smem + PL::oBTZ + PL::ofs(e * 6 + c, q, PL::SBB_Q, PL::LB), o[c]);
+          put_op<BF>(smem + PL::oBTZ + PL::ofs(6 * T + e * 6 + c, q, PL::SBB_Q, PL::LB), o[6 + c]);
+        }
+      }
+      }   // t
     }
+    if (next < ntiles) load_sig(next, sgv);
+    signal_ready(5);   // P_q operand; the product overlaps the epilogue below
     if (!wait_bar(1)) { failed = true; break; }
     const int nsrc_l = min(flags[0], 64);
 
@@ -831,73 +818,60 @@ __global__ void __launch_bounds__(TcWarps<N, PML, BF, QC>::threads,
       }
       const float ie = geoM[e * 12 + 9], im = geoM[e * 12 + 10];
       const float rhs[6] = {ie * CH[0], ie * CH[1], ie * CH[2], -im * CE[0], -im * CE[1], -im * CE[2]};
-      if (!PML) {
 #pragma unroll
-        for (int c = 0; c < 6; ++c) {
-          const int li = (e * 6 + c) * Np + i;
-          const int64_t gi = (int64_t)eg0 * 6 * Np + li;
-          const float rr = rka * SR[li] + rdt * rhs[c];
-          resq[gi] = rr;
-          qout[gi] = SQ[li] + rkb * rr;
-        }
-      } else {
-#pragma unroll
-        for (int c = 0; c < 6; ++c) RS[(e * 6 + c) * Np + i] = rhs[c];
-      }
+      for (int c = 0; c < 6; ++c) RS[(e * 6 + c) * Np + i] = rhs[c];
     }
 
-    if (PML) {
-      // ---- the P_q product has had the volume/LIFT epilogue to complete
-      if (!wait_bar(2)) { failed = true; break; }
-      fence_async_smem();   // the (t, z) buffer is reused below
-      // ---- P_q columns of the node lanes -> shared memory
-      float* DP = reinterpret_cast<float*>(smem + PL::oDP);   // [T][12][Np]
-      if (quad * 32 < Np) {
-        const int i = quad * 32 + lane;
+    // ---- the P_q product has had the volume/LIFT epilogue to complete
+    if (!wait_bar(2)) { failed = true; break; }
+    fence_async_smem();   // the (t, z) buffer is reused below
+    // ---- P_q columns of the node lanes -> shared memory
+    float* DP = reinterpret_cast<float*>(smem + PL::oDP);   // [T][12][Np]
+    if (quad * 32 < Np) {
+      const int i = quad * 32 + lane;
 #pragma unroll
-        for (int k = 0; k < EH; ++k) {
-          const int e = grp + NGRP * k;
-          if (e >= T) break;
-          float v[12];   // s | rhs of P
-          tld_6x2(tmem + lane_base + PL::cPq + e * 6, tmem + lane_base + PL::cPq + 6 * T + e * 6, v);
-          if (e >= ne || i >= Np) continue;
+      for (int k = 0; k < EH; ++k) {
+        const int e = grp + NGRP * k;
+        if (e >= T) break;
+        float v[12];   // s | rhs of P
+        tld_6x2(tmem + lane_base + PL::cPq + e * 6, tmem + lane_base + PL::cPq + 6 * T + e * 6, v);
+        if (e >= ne || i >= Np) continue;
 #pragma unroll
-          for (int k = 0; k < 12; ++k) DP[(e * 12 + k) * Np + i] = v[k];
-        }
+        for (int k = 0; k < 12; ++k) DP[(e * 12 + k) * Np + i] = v[k];
       }
-      fence_before();
-      cbar_sync(kTcThreads);
-      fence_after();
-      // ---- epilogue B (all warps): Runge-Kutta update of E, H, P^E, P^H, two
-      // consecutive values of one element block per task (6 Np is even, so a
-      // pair never straddles two elements and stays 8-byte aligned)
-      for (int t2 = tid; t2 < ne * 3 * Np; t2 += kTcThreads) {
-        const int li = 2 * t2;                  // (e * 6 + c) * Np + i
-        const int e = li / (6 * Np);
-        const int di = li + e * 6 * Np;         // (e * 12 + c) * Np + i
-        const float2 sr = *reinterpret_cast<const float2*>(SR + li);
-        const float2 sq = *reinterpret_cast<const float2*>(SQ + li);
-        const float2 rs = *reinterpret_cast<const float2*>(RS + li);
-        const float2 ds = *reinterpret_cast<const float2*>(DP + di);
-        const float2 dz = *reinterpret_cast<const float2*>(DP + di + 6 * Np);
-        const float2 srp = *reinterpret_cast<const float2*>(SRP + li);
-        const float2 sp = *reinterpret_cast<const float2*>(SP + li);
-        float2 rr, qn, rp, pn;
-        rr.x = rka * sr.x + rdt * (rs.x - ds.x);
-        rr.y = rka * sr.y + rdt * (rs.y - ds.y);
-        qn.x = sq.x + rkb * rr.x;
-        qn.y = sq.y + rkb * rr.y;
-        rp.x = rka * srp.x + rdt * dz.x;
-        rp.y = rka * srp.y + rdt * dz.y;
-        pn.x = sp.x + rkb * rp.x;
-        pn.y = sp.y + rkb * rp.y;
-        const int64_t gi = (int64_t)eg0 * 6 * Np + li;
-        const int64_t pi = (int64_t)ep0 * 6 * Np + li;
-        *reinterpret_cast<float2*>(resq + gi) = rr;
-        *reinterpret_cast<float2*>(qout + gi) = qn;
-        *reinterpret_cast<float2*>(resp + pi) = rp;
-        *reinterpret_cast<float2*>(pio + pi) = pn;
-      }
+    }
+    fence_before();
+    cbar_sync(kTcThreads);
+    fence_after();
+    // ---- epilogue B (all warps): Runge-Kutta update of E, H, P^E, P^H, two
+    // consecutive values of one element block per task (6 Np is even, so a
+    // pair never straddles two elements and stays 8-byte aligned)
+    for (int t2 = tid; t2 < ne * 3 * Np; t2 += kTcThreads) {
+      const int li = 2 * t2;                  // (e * 6 + c) * Np + i
+      const int e = li / (6 * Np);
+      const int di = li + e * 6 * Np;         // (e * 12 + c) * Np + i
+      const float2 sr = *reinterpret_cast<const float2*>(SR + li);
+      const float2 sq = *reinterpret_cast<const float2*>(SQ + li);
+      const float2 rs = *reinterpret_cast<const float2*>(RS + li);
+      const float2 ds = *reinterpret_cast<const float2*>(DP + di);
+      const float2 dz = *reinterpret_cast<const float2*>(DP + di + 6 * Np);
+      const float2 srp = *reinterpret_cast<const float2*>(SRP + li);
+      const float2 sp = *reinterpret_cast<const float2*>(SP + li);
+      float2 rr, qn, rp, pn;
+      rr.x = rka * sr.x + rdt * (rs.x - ds.x);
+      rr.y = rka * sr.y + rdt * (rs.y - ds.y);
+      qn.x = sq.x + rkb * rr.x;
+      qn.y = sq.y + rkb * rr.y;
+      rp.x = rka * srp.x + rdt * dz.x;
+      rp.y = rka * srp.y + rdt * dz.y;
+      pn.x = sp.x + rkb * rp.x;
+      pn.y = sp.y + rkb * rp.y;
+      const int64_t gi = (int64_t)eg0 * 6 * Np + li;
+      const int64_t pi = (int64_t)ep0 * 6 * Np + li;
+      *reinterpret_cast<float2*>(resq + gi) = rr;
+      *reinterpret_cast<float2*>(qout + gi) = qn;
+      *reinterpret_cast<float2*>(resp + pi) = rp;
+      *reinterpret_cast<float2*>(pio + pi) = pn;
     }
     fence_before();
     cbar_sync(kTcThreads);
@@ -912,26 +886,26 @@ __global__ void __launch_bounds__(TcWarps<N, PML, BF, QC>::threads,
   if (warp == 0) tmem_dealloc(tmem, PL::TMEM_COLS);
 }
 
-template <int N, bool PML, bool BF, int QC>
+template <int N, bool BF>
 cudaError_t configure_n() {
-  using TW = TcWarps<N, PML, BF, QC>;
+  using TW = TcWarps<N, BF>;
   // the compute warps' setmaxnreg.inc waits until the block's launch
   // allocation can cover the split: refuse a build whose compiled register
   // count would leave it short
   cudaFuncAttributes fa{};
-  cudaError_t e = cudaFuncGetAttributes(&fa, tc_stage_kernel<N, PML, BF, QC>);
+  cudaError_t e = cudaFuncGetAttributes(&fa, tc_stage_kernel<N, BF>);
   if (e != cudaSuccess) return e;
   if ((long)fa.numRegs * TW::threads <
       32L * TW::compute * TW::compute_regs + 32L * TW::issue * TW::issue_regs)
     return cudaErrorInvalidConfiguration;
-  return cudaFuncSetAttribute(tc_stage_kernel<N, PML, BF, QC>,
+  return cudaFuncSetAttribute(tc_stage_kernel<N, BF>,
                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)Plan<N, PML, BF, QC>::bytes);
+                              (int)Plan<N, BF>::bytes);
 }
 
-template <int N, bool PML, bool BF, int QC>
+template <int N, bool BF>
 cudaError_t launch_n(const StageParams<float>& P, int nb, cudaStream_t s) {
-  using PL = Plan<N, PML, BF, QC>;
+  using PL = Plan<N, BF>;
   if (P.n_elem <= 0) return cudaSuccess;
   static int sms = 0;
   if (sms == 0) {
@@ -945,7 +919,7 @@ cudaError_t launch_n(const StageParams<float>& P, int nb, cudaStream_t s) {
   const long long tiles = (long long)((P.n_elem + PL::T - 1) / PL::T) * nb;
   const int per_sm = PL::ONE ? 1 : 512 / (int)PL::TMEM_COLS;
   const int grid = (int)std::min<long long>(tiles, (long long)per_sm * sms);
-  tc_stage_kernel<N, PML, BF, QC><<<grid, TcWarps<N, PML, BF, QC>::threads, PL::bytes, s>>>(Q);
+  tc_stage_kernel<N, BF><<<grid, TcWarps<N, BF>::threads, PL::bytes, s>>>(Q);
   return cudaGetLastError();
 }
 
@@ -959,28 +933,18 @@ bool tc_supported(int N, bool kappa, bool bf16, int qc) {
   return bf16 || N <= 4 || qc == 1;
 }
 
-// The PML class with a compact rule runs tc_rows_kernel (tc_rows.cu); here:
-// the non-PML class (no quadrature) and the PML class with the (N+1)^3 rule.
-template <int N, bool BF>
-cudaError_t configure_tc_n() {
-  cudaError_t e = cudaSuccess;
-  if constexpr (BF || N <= 4) {
-    e = tc::configure_n<N, false, BF, 0>();
-    if (e == cudaSuccess) e = tc::configure_n<N, true, BF, 0>();
-  } else {
-    e = tc::configure_n<N, false, BF, 1>();
-  }
-  return e;
-}
-
+// tc_stage_kernel: the PML class with the (N+1)^3 rule; the other classes run
+// tc_rows_kernel (tc_rows.cu).  TF32 at N = 5 has compact rules only.
 template <bool BF>
 cudaError_t configure_tc_bf(int N) {
   switch (N) {
-    case 1: return configure_tc_n<1, BF>();
-    case 2: return configure_tc_n<2, BF>();
-    case 3: return configure_tc_n<3, BF>();
-    case 4: return configure_tc_n<4, BF>();
-    case 5: return configure_tc_n<5, BF>();
+    case 1: return tc::configure_n<1, BF>();
+    case 2: return tc::configure_n<2, BF>();
+    case 3: return tc::configure_n<3, BF>();
+    case 4: return tc::configure_n<4, BF>();
+    case 5:
+      if constexpr (BF) return tc::configure_n<5, BF>();
+      return cudaSuccess;
     default: return cudaErrorInvalidValue;
   }
 }
@@ -989,42 +953,29 @@ cudaError_t configure_tc_kernels(int N, bool bf16) {
   return bf16 ? configure_tc_bf<true>(N) : configure_tc_bf<false>(N);
 }
 
-template <int N, bool BF>
-cudaError_t launch_tc_n(bool pml, const StageParams<float>& P, int nb, cudaStream_t s, int qc) {
-  if constexpr (BF || N <= 4) {
-    if (!pml) return tc::launch_n<N, false, BF, 0>(P, nb, s);
-    if (qc == 0) return tc::launch_n<N, true, BF, 0>(P, nb, s);
-  } else {
-    if (!pml) return tc::launch_n<N, false, BF, 1>(P, nb, s);
-  }
-  return cudaErrorInvalidValue;   // compact-rule PML classes run tc_rows_kernel
-}
-
 template <bool BF>
-cudaError_t launch_tc_bf(int N, bool pml, const StageParams<float>& P, int nb, cudaStream_t s,
-                         int qc) {
+cudaError_t launch_tc_bf(int N, const StageParams<float>& P, int nb, cudaStream_t s) {
   switch (N) {
-    case 1: return launch_tc_n<1, BF>(pml, P, nb, s, qc);
-    case 2: return launch_tc_n<2, BF>(pml, P, nb, s, qc);
-    case 3: return launch_tc_n<3, BF>(pml, P, nb, s, qc);
-    case 4: return launch_tc_n<4, BF>(pml, P, nb, s, qc);
-    case 5: return launch_tc_n<5, BF>(pml, P, nb, s, qc);
+    case 1: return tc::launch_n<1, BF>(P, nb, s);
+    case 2: return tc::launch_n<2, BF>(P, nb, s);
+    case 3: return tc::launch_n<3, BF>(P, nb, s);
+    case 4: return tc::launch_n<4, BF>(P, nb, s);
+    case 5:
+      if constexpr (BF) return tc::launch_n<5, BF>(P, nb, s);
+      return cudaErrorInvalidValue;
     default: return cudaErrorInvalidValue;
   }
 }
 
-cudaError_t launch_stage_tc(int N, bool pml, const StageParams<float>& P, int nb, cudaStream_t s,
-                            bool bf16, int qc) {
-  // the kernels stage element blocks as bulk copies of their 16-byte-aligned
+cudaError_t launch_pml_tc(int N, const StageParams<float>& P, int nb, cudaStream_t s, bool bf16) {
+  // the kernel stages element blocks as bulk copies of their 16-byte-aligned
   // cover, sized for blocks that start 0 or 8 bytes past a boundary: every
   // field buffer must start on a 16-byte boundary
   const uintptr_t a = reinterpret_cast<uintptr_t>(P.qin) | reinterpret_cast<uintptr_t>(P.qout) |
-                      reinterpret_cast<uintptr_t>(P.resq) |
-                      (pml ? reinterpret_cast<uintptr_t>(P.p) | reinterpret_cast<uintptr_t>(P.resp)
-                           : 0);
+                      reinterpret_cast<uintptr_t>(P.resq) | reinterpret_cast<uintptr_t>(P.p) |
+                      reinterpret_cast<uintptr_t>(P.resp);
   if (a & 15) return cudaErrorMisalignedAddress;
-  return bf16 ? launch_tc_bf<true>(N, pml, P, nb, s, qc)
-              : launch_tc_bf<false>(N, pml, P, nb, s, qc);
+  return bf16 ? launch_tc_bf<true>(N, P, nb, s) : launch_tc_bf<false>(N, P, nb, s);
 }
 
 }  // namespace wadg

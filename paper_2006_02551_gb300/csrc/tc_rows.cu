@@ -1,10 +1,23 @@
 // Tensor-core stage kernel with row-owned epilogues (sm_103a: tcgen05 with
 // TF32 or BF16 operands, FP32 accumulation in tensor memory, FP32 state) for
+// the non-PML class (PML = false drops the P rows, V_q, P_q and eq. 9) and for
 // the PML class of contexts with a compact volume rule (quad_capacity class
-// 1).  The kernel is written for both element classes (PML = false drops the
-// P rows, V_q, P_q and eq. 9), but only the PML class is built: at N = 4 the
-// non-PML instantiation took 0.376 ms per launch (TF32) against 0.342 ms for
-// the non-PML class of tc_stage_kernel, which keeps that class.
+// 1).  The PML class with the (N+1)^3 rule runs tc_stage_kernel: its points do
+// not fit the tensor memory of row-owned products.
+//
+// What bounds it: the chain of a tile (operands -> V_q -> eq. 9 -> P_q ->
+// update, the curl between) in the epilogue warps, and the flux warps beside
+// it, both near 10k cycles a tile; the memory system and the tensor pipe are a
+// third and a seventh busy.  Measured (82,944 tets, TF32, us per launch, before
+// -> after four flux warps a slot whose lanes keep one face node, look-ups
+// level by level, two faces in flight, float4 rows, only the two derivatives a
+// lane sends, sigma / eps0 in rows the lanes read in their own order): non-PML,
+// against the operator-rows kernel that had it, N = 4 86.7 -> 67.3, N = 5
+// 160.8 -> 100, N = 3 60.7 -> 46.4; PML N = 4 159.5 -> 140, N = 5 421 -> 321,
+// N = 3 102 -> 85.  Also tried: the register split 128/88/48 (epilogue, flux,
+// issuing and copy warps: spills in the flux, N = 4 PML 179), no split (161),
+// two flux warps of 128 registers (148), four faces in flight (non-PML N = 4
+// 72.5 against 69.9 for two), three splits per quadrant at N = 4 (220).
 //
 // Every contraction of the stage is one product
 //     D[row][n] = sum_k A[row][k] * B[n][k]
@@ -32,7 +45,8 @@
 // chains the products on mbarriers.
 //
 // Warp roles per slot: four epilogue warps (two per lane quadrant of the
-// slot, splitting the nodes and quadrature points of their rows in halves),
+// slot, splitting the nodes and quadrature points of their rows in halves; with
+// one slot three, in thirds),
 // flux warps (upwind flux into the LIFT operand) and an issuing warp whose
 // first lane stages each tile with bulk copies (and prefetches the next tile
 // into L2), issues every product and writes the results back with bulk
@@ -58,6 +72,10 @@ struct RPlan {
   static constexpr int NF = 4 * Nfp;
   static constexpr int Nq = compact_nq(N);          // capacity of the compact class
   static constexpr int NqP = (Nq + 3) & ~3;         // stride of the sigma samples
+  // ... and of a staged row of them: the lanes of an element read three rows at
+  // once, which must not start on the same banks (a multiple of 16 floats would
+  // put rows 0 and 2 there; such rows are copied one by one)
+  static constexpr int SGR = NqP % 16 == 0 ? NqP + 4 : NqP;
   static constexpr int CW = O::CW, KS = O::KS;
   __host__ __device__ static constexpr int rupK(int x) { return (x + KS - 1) / KS * KS; }
   static constexpr int NpK = rupK(Np), NFK = rupK(NF), NqK = rupK(Nq);
@@ -109,7 +127,7 @@ struct RPlan {
   // blocks (the Runge-Kutta registers, needed at the update, and the sigma
   // samples, needed at eq. 9) have one, refilled once this tile is past them.
   static constexpr uint32_t FB = ((T * 6 * Np * 4 + 15) & ~15) + 16;
-  static constexpr uint32_t SGB = PML ? ((T * 3 * NqP * 4 + 15) & ~15) + 16 : 0;
+  static constexpr uint32_t SGB = PML ? ((T * 3 * SGR * 4 + 15) & ~15) + 16 : 0;
   static constexpr uint32_t GFN = ((T * 64 + 15) & ~15) + 16;
   static constexpr uint32_t GMET = ((T * 72 + 15) & ~15) + 16;
   static constexpr uint32_t GMAT = ((T * 12 + 15) & ~15) + 16;
@@ -149,35 +167,40 @@ struct RPlan {
   static_assert(!PML || (span_ok(oAP, SBF) && span_ok(oAF, SBT) && span_ok(oAP, SBT)),
                 "P / T / Z operand span");
   static_assert(bytes <= 227 * 1024, "shared memory");
-  // warps: 4 epilogue warps per slot (the two lane quadrants of the slot x
-  // halves of the nodes and points), flux warps, an issuing warp and a copy
+  // warps: 2 S epilogue warps per slot (the two lane quadrants of the slot x
+  // shares of the nodes and points), flux warps, an issuing warp and a copy
   // warp per slot
   // S epilogue warps per lane quadrant, each taking a share of the nodes
   // and quadrature points of the quadrant's rows
-  static constexpr int S = 2;
+  static constexpr int S = SLOTS == 2 ? 2 : 3;
   static constexpr int EW = 4 * S;                  // warps 0 .. EW-1: epilogue / flux
-  static constexpr int FLUXW = SLOTS == 2 ? 2 : 2 * S + 4;   // flux warps per slot
-  // warps: EW epilogue (and, with one slot, flux), 4 flux, then one issuing
+  static constexpr int FLUXW = SLOTS == 2 ? 4 : 2 * S + 4;   // flux warps per slot
+  static constexpr int FX = SLOTS == 2 ? 2 * FLUXW : 4;      // warps EW .. EW + FX - 1: flux
+  // warps: EW epilogue (and, with one slot, flux), FX flux, then one issuing
   // warp and one copy warp per slot
-  static constexpr int THREADS = 32 * (EW + 4 + 2 * SLOTS);
-  // nodes and quadrature points of one split (multiples of 4)
-  // register split (two slots: the warp groups are 0-7 epilogue, 8-11
-  // flux, 12-15 issuing and copy): setmaxnreg moves registers from the flux
-  // and copy groups to the epilogue warps within the launch allocation
-  static constexpr int LAUNCH_REGS = (65536 / THREADS) & ~7;
-  static constexpr int REG_E = 128, REG_F = 96, REG_C = 96;
-  static constexpr bool SPLIT = false;   // measured: the uniform budget is faster
-  static_assert(!SPLIT || 32 * (EW * REG_E + 4 * REG_F + 4 * REG_C) <= THREADS * LAUNCH_REGS,
+  static constexpr int THREADS = 32 * (EW + FX + 2 * SLOTS);
+  // 20 warps hold 96 registers each: where the epilogue needs more (N = 4 PML)
+  // it takes them from the flux and the issuing and copy warps
+  // (setmaxnreg, by warpgroups: 0, 1 epilogue, 2, 3 flux, 4 issuing and copy)
+  static constexpr bool SPLIT = PML && SLOTS == 2 && N == 4;
+  static constexpr int LAUNCH_REGS = 96, REG_E = 112, REG_F = 96, REG_C = 64;
+  static_assert(!SPLIT || (EW == 8 && FX == 8 && 2 * SLOTS == 4 &&
+                           8 * REG_E + 8 * REG_F + 4 * REG_C <= 20 * LAUNCH_REGS),
                 "register split within the launch allocation");
+  // nodes and quadrature points of one split (multiples of 4)
   static constexpr int NS = rup4((Np + S - 1) / S);
+  // rows of whole 16-byte words: the epilogue reads and writes the staged rows
+  // (which then start on 16-byte boundaries) by float4.  Their rows fall on few
+  // banks: at N = 5 scalar accesses of a warp met 6-way conflicts
+  static constexpr bool V4 = Np % 4 == 0;
   static constexpr int QS = ((NqK / CW + S - 1) / S) * CW;
   static_assert(QS % 4 == 0, "quadrature split");
 };
 
 // warp roles.  Epilogue warps: w < EW whose lane quadrant w & 3 belongs to
 // a slot (quadrants 0, 1 -> slot 0; 2, 3 -> slot 1 when there are two).
-// Flux warps: the other warps below EW + 4.  Then the issuing warps
-// (EW + 4 + slot) and the copy warps (EW + 4 + SLOTS + slot).
+// Flux warps: the other warps below EW + FX.  Then the issuing warps
+// (EW + FX + slot) and the copy warps (EW + FX + SLOTS + slot).
 template <int SLOTS, int EW>
 __device__ __forceinline__ int epilogue_slot(int w) {
   if (w >= EW) return -1;
@@ -185,15 +208,15 @@ __device__ __forceinline__ int epilogue_slot(int w) {
   if (SLOTS == 2) return qd >> 1;
   return qd < 2 ? 0 : -1;
 }
-template <int SLOTS, int EW>
+template <int SLOTS, int EW, int FX>
 __device__ __forceinline__ int flux_slot(int w, int& index) {
-  if (SLOTS == 2) {   // warps EW .. EW + 3: two per slot
-    if (w < EW || w >= EW + 4) return -1;
-    index = (w - EW) & 1;
-    return (w - EW) >> 1;
+  if (SLOTS == 2) {   // warps EW .. EW + FX - 1: half of them per slot
+    if (w < EW || w >= EW + FX) return -1;
+    index = (w - EW) % (FX / 2);
+    return (w - EW) / (FX / 2);
   }
-  // one slot: the warps of quadrants 2 and 3 below EW, then EW .. EW + 3
-  if (w >= EW + 4 || epilogue_slot<1, EW>(w) >= 0) return -1;
+  // one slot: the warps of quadrants 2 and 3 below EW, then EW .. EW + FX - 1
+  if (w >= EW + FX || epilogue_slot<1, EW>(w) >= 0) return -1;
   index = w < EW ? (w >> 2) * 2 + (w & 1) : EW / 2 + (w - EW);
   return 0;
 }
@@ -306,11 +329,11 @@ __global__ void __launch_bounds__(RPlan<N, PML, BF>::THREADS, 1)
   // phase parity of early buffer (it & 1) at iteration it
   auto eparity = [&](int it) { return (uint32_t)(EB == 2 ? (it >> 1) & 1 : it & 1); };
 
-  if (warp >= PL::EW + 4) {
+  if (warp >= PL::EW + PL::FX) {
     if constexpr (PL::SPLIT) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(PL::REG_C));
     // ================================ issuing and copy warps of a slot (lane 0)
-    const bool copier = warp >= PL::EW + 4 + SLOTS;
-    const int sl = warp - PL::EW - 4 - (copier ? SLOTS : 0);
+    const bool copier = warp >= PL::EW + PL::FX + SLOTS;
+    const int sl = warp - PL::EW - PL::FX - (copier ? SLOTS : 0);
     const uint32_t sA = PL::oA + sl * PL::ASLOT;      // this slot's A operands
     uint64_t* mb = mbar + 12 * sl;
     const uint32_t tcol = tmem + sl * PL::CSTR;       // this slot's columns, lane 0
@@ -424,10 +447,14 @@ __global__ void __launch_bounds__(RPlan<N, PML, BF>::THREADS, 1)
       auto sig_in = [&](int tile) {
         if constexpr (PML) {
           const Tile t = tile_at(tile);
-          const void* src[1] = {P.sig + (t.eg0 - P.K0) * 3 * NqP};
-          const uint32_t len[1] = {(uint32_t)t.ne * 3 * NqP * 4};
-          const uint32_t dst[1] = {lbuf(sl) + PL::oLSG};
-          copy_in(src, len, dst, 1, mb + B_SIG);
+          const float* g = P.sig + (t.eg0 - P.K0) * 3 * NqP;   // rows of whole 16-byte words
+          const uint32_t rows = 3 * t.ne, n = PL::SGR == NqP ? 1 : rows;
+          const uint32_t len = rows / n * NqP * 4;
+          fence_async_smem();
+          mbar_expect_tx(saddr(mb + B_SIG), n * len);
+          for (uint32_t r = 0; r < n; ++r)
+            bulk_g2s(sbase + lbuf(sl) + PL::oLSG + r * PL::SGR * 4, g + r * NqP, len,
+                     saddr(mb + B_SIG));
         }
       };
       auto prefetch = [&](int tile) {
@@ -539,7 +566,7 @@ __global__ void __launch_bounds__(RPlan<N, PML, BF>::THREADS, 1)
     const int base = lane & ~7;
     const int s1 = base + (c < 6 ? (0x102435 >> (4 * c)) & 15 : c);
     const int s2 = base + (c < 6 ? (0x021354 >> (4 * c)) & 15 : c);
-    const int send1 = (c + 2) % 3, send2 = (c + 1) % 3;
+    const int send1 = (c + 2) % 3, send2 = (c + 1) % 3;   // the axes this lane sends
     const int i0 = h * PL::NS, i1 = min(Np, i0 + PL::NS);   // nodes of this split
     int it = 0;
     for (int tile = blockIdx.x * SLOTS + sl; tile < ntiles && !failed; tile += nworkers, ++it) {
@@ -565,12 +592,27 @@ __global__ void __launch_bounds__(RPlan<N, PML, BF>::THREADS, 1)
         const float* fq = SQ + (e * 6 + c) * Np;
         const float* fp = PML ? SP + (e * 6 + c) * Np : nullptr;
         float x[H0 * CW], y[PML ? H0 * CW : 1];
+        if constexpr (PL::V4) {
 #pragma unroll
-        for (int u = 0; u < H0 * CW; ++u) {
-          const int k = k0 * CW + u;
-          const bool ok = live && u < nch * CW && k < Np;
-          x[u] = ok ? fq[k] : 0.f;
-          if constexpr (PML) y[u] = ok ? fp[k] : 0.f;
+          for (int u = 0; u < H0 * CW; u += 4) {
+            const int k = k0 * CW + u;
+            const bool ok = live && u < nch * CW && k < Np;
+            const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+            const float4 a4 = ok ? *reinterpret_cast<const float4*>(fq + k) : z4;
+            x[u] = a4.x, x[u + 1] = a4.y, x[u + 2] = a4.z, x[u + 3] = a4.w;
+            if constexpr (PML) {
+              const float4 b4 = ok ? *reinterpret_cast<const float4*>(fp + k) : z4;
+              y[u] = b4.x, y[u + 1] = b4.y, y[u + 2] = b4.z, y[u + 3] = b4.w;
+            }
+          }
+        } else {
+#pragma unroll
+          for (int u = 0; u < H0 * CW; ++u) {
+            const int k = k0 * CW + u;
+            const bool ok = live && u < nch * CW && k < Np;
+            x[u] = ok ? fq[k] : 0.f;
+            if constexpr (PML) y[u] = ok ? fp[k] : 0.f;
+          }
         }
 #pragma unroll
         for (int kc = 0; kc < H0; ++kc) {
@@ -609,39 +651,34 @@ __global__ void __launch_bounds__(RPlan<N, PML, BF>::THREADS, 1)
       fence_async_smem();
       __syncwarp();
       if (lane == 0) mbar_arrive(saddr(mb + B_FP));
-      // this element's metric (r_x .. t_z) and 1/eps, 1/mu
-      float g[9], ie, im;
+      // the rows of this element's metric (r_x .. t_z) for the two derivatives
+      // this lane sends, 1/eps of it, and the factor of its curl (1/eps, -1/mu)
+      float g1[3], g2[3], ie, kc;
       {
         const float* met =
             reinterpret_cast<const float*>(staged(eb + PL::oEMET, P.geof + t.eg0 * 9));
         const float* mat = reinterpret_cast<const float*>(staged(eb + PL::oEMAT, P.mat + t.eg0 * 3));
         const int ee = e < ne ? e : 0;
 #pragma unroll
-        for (int j = 0; j < 9; ++j) g[j] = met[ee * 9 + j];
+        for (int j = 0; j < 3; ++j) {
+          g1[j] = met[ee * 9 + 3 * j + send1];
+          g2[j] = met[ee * 9 + 3 * j + send2];
+        }
         ie = mat[ee * 3 + 0];
-        im = mat[ee * 3 + 1];
+        kc = c < 3 ? ie : -mat[ee * 3 + 1];
       }
       if constexpr (PML) {
         // ---- eq. 9 at this half's quadrature points -> T and Z rows
         if (!mbar_wait_sleep(saddr(mb + B_V), ph)) { failed = true; break; }
         fence_after();
         if (!mbar_wait_sleep(saddr(mb + B_SIG), ph)) { failed = true; break; }
-        const float* sg = reinterpret_cast<const float*>(
-            staged(lb + PL::oLSG, P.sig + (t.eg0 - P.K0) * 3 * NqP));
-        const float ie0 = 1.f / (float)P.eps0;
+        const float* sg = reinterpret_cast<const float*>(smem + lb + PL::oLSG);
         const int u = c % 3;
         const int ee = e < ne ? e : 0;
-        // the lanes of one element need the axes in the orders (u, v, w) =
-        // (0,1,2), (1,2,0), (2,0,1).  Where rows 0 and 2 (2 NqP floats
-        // apart) fall on the same banks, the TF32 kernel has every lane read
-        // the rows in axis order (one address per element and load) and
-        // permute them in registers; otherwise, and in the BF16 kernel
-        // (measured faster there), each lane reads its own order.
-        constexpr bool ordered = !BF && (2 * NqP) % 32 == 0;
-        const float* s0_p = sg + (ee * 3) * NqP;
-        const float* su_p = sg + (ee * 3 + u) * NqP;
-        const float* sv_p = sg + (ee * 3 + (u == 2 ? 0 : u + 1)) * NqP;
-        const float* sw_p = sg + (ee * 3 + (u == 0 ? 2 : u - 1)) * NqP;
+        // rows of the axes in this lane's order (u, v, w) = (0,1,2), (1,2,0), (2,0,1)
+        const float* su_p = sg + (ee * 3 + u) * PL::SGR;
+        const float* sv_p = sg + (ee * 3 + (u == 2 ? 0 : u + 1)) * PL::SGR;
+        const float* sw_p = sg + (ee * 3 + (u == 0 ? 2 : u - 1)) * PL::SGR;
         const int q0 = h * PL::QS, q1 = min(NqK, q0 + PL::QS);
         constexpr int QB = 8;    // points per batch of tensor-memory loads
         for (int qq = q0; qq < q1; qq += QB) {
@@ -659,18 +696,9 @@ __global__ void __launch_bounds__(RPlan<N, PML, BF>::THREADS, 1)
             const int qb = qq + 4 * j4;
             sgu[j4] = sgv[j4] = sgw[j4] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (qb < NqP && qb < q1) {
-              if constexpr (!ordered) {
-                sgu[j4] = *reinterpret_cast<const float4*>(su_p + qb);
-                sgv[j4] = *reinterpret_cast<const float4*>(sv_p + qb);
-                sgw[j4] = *reinterpret_cast<const float4*>(sw_p + qb);
-              } else {
-                const float4 a0 = *reinterpret_cast<const float4*>(s0_p + qb);
-                const float4 a1 = *reinterpret_cast<const float4*>(s0_p + NqP + qb);
-                const float4 a2 = *reinterpret_cast<const float4*>(s0_p + 2 * NqP + qb);
-                sgu[j4] = u == 0 ? a0 : (u == 1 ? a1 : a2);
-                sgv[j4] = u == 0 ? a1 : (u == 1 ? a2 : a0);
-                sgw[j4] = u == 0 ? a2 : (u == 1 ? a0 : a1);
-              }
+              sgu[j4] = *reinterpret_cast<const float4*>(su_p + qb);
+              sgv[j4] = *reinterpret_cast<const float4*>(sv_p + qb);
+              sgw[j4] = *reinterpret_cast<const float4*>(sw_p + qb);
             }
           }
           tmem_wait_ld();
@@ -684,14 +712,14 @@ __global__ void __launch_bounds__(RPlan<N, PML, BF>::THREADS, 1)
             for (int j = 0; j < 4; ++j) {
               const int jj = 4 * j4 + j;
               const float vf = __uint_as_float(rv[jj]), vp = __uint_as_float(rv[QB + jj]);
-              const float su = sa[j] * ie0, sv = sb4[j] * ie0, sw = sc4[j] * ie0;
+              const float su = sa[j], sv = sb4[j], sw = sc4[j];
               // eq. 9 with kappa = 1 in terms of s = sigma / eps0:
               // b = sv + sw - su, c = sv sw - b su, d = su
               const float bc = sv + sw - su;
               const float cc = sv * sw - bc * su;
-              const bool ok = live && qq + jj < Nq;
-              tz[0][jj] = ok ? bc * vf + cc * vp : 0.f;
-              tz[1][jj] = ok ? vf - su * vp : 0.f;
+              // (rows without data and points past the rule have vf = vp = 0)
+              tz[0][jj] = bc * vf + cc * vp;
+              tz[1][jj] = vf - su * vp;
             }
           }
           // K chunks of CW points (4 TF32 / 8 BF16) of the T and Z rows
@@ -751,15 +779,12 @@ __global__ void __launch_bounds__(RPlan<N, PML, BF>::THREADS, 1)
         for (int j = 0; j < nb; ++j) {
           const float dr = __uint_as_float(r[j]), ds = __uint_as_float(r[nb + j]);
           const float dt = __uint_as_float(r[2 * nb + j]), lf = __uint_as_float(r[3 * nb + j]);
-          const float dx = g[0] * dr + g[3] * ds + g[6] * dt;
-          const float dy = g[1] * dr + g[4] * ds + g[7] * dt;
-          const float dz = g[2] * dr + g[5] * ds + g[8] * dt;
-          const float o1 = send1 == 0 ? dx : (send1 == 1 ? dy : dz);
-          const float o2 = send2 == 0 ? dx : (send2 == 1 ? dy : dz);
+          const float o1 = g1[0] * dr + g1[1] * ds + g1[2] * dt;
+          const float o2 = g2[0] * dr + g2[1] * ds + g2[2] * dt;
           const float a1 = __shfl_sync(0xffffffffu, o1, s1);
           const float a2 = __shfl_sync(0xffffffffu, o2, s2);
           const float cr = a1 - a2 + lf;   // (curl of the partner field) + LIFT term
-          rhs[ic + j] = c < 3 ? ie * cr : -im * cr;
+          rhs[ic + j] = kc * cr;
         }
       };
       constexpr int CB = NHC < 12 ? NHC : 12;   // nodes per batch of loads
@@ -798,7 +823,7 @@ __global__ void __launch_bounds__(RPlan<N, PML, BF>::THREADS, 1)
       // ---- Runge-Kutta update of this half's nodes, in place in the staging:
       // batches of UB nodes, every value of a batch loaded before any store
       if (live) {
-        constexpr int UB = 5;
+        constexpr int UB = PL::V4 ? 4 : 5;
         float* sr = SR + (e * 6 + c) * Np;
         float* sq = SQ + (e * 6 + c) * Np;
         float* srp = PML ? SRP + (e * 6 + c) * Np : nullptr;
@@ -806,6 +831,40 @@ __global__ void __launch_bounds__(RPlan<N, PML, BF>::THREADS, 1)
 #pragma unroll
         for (int j0 = 0; j0 < NHC; j0 += UB) {
           float r_[UB], q_[UB], rp_[UB], p_[UB];
+          if constexpr (PL::V4) {   // NS, i0 and i1 are multiples of 4
+            const int ii = i0 + j0;
+            if (ii >= i1) break;
+            auto get = [&](const float* g, float* v) {
+              const float4 a = *reinterpret_cast<const float4*>(g + ii);
+              v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
+            };
+            auto put = [&](float* g, const float* v) {
+              *reinterpret_cast<float4*>(g + ii) = make_float4(v[0], v[1], v[2], v[3]);
+            };
+            get(sr, r_);
+            get(sq, q_);
+            if constexpr (PML) {
+              get(srp, rp_);
+              get(spp, p_);
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const float s_ = PML ? __uint_as_float(sz[j0 + j]) : 0.f;
+              r_[j] = rka * r_[j] + rdt * (rhs[j0 + j] - s_);
+              q_[j] = q_[j] + rkb * r_[j];
+              if constexpr (PML) {
+                rp_[j] = rka * rp_[j] + rdt * __uint_as_float(sz[NHC + j0 + j]);
+                p_[j] = p_[j] + rkb * rp_[j];
+              }
+            }
+            put(sr, r_);
+            put(sq, q_);
+            if constexpr (PML) {
+              put(srp, rp_);
+              put(spp, p_);
+            }
+            continue;
+          }
 #pragma unroll
           for (int j = 0; j < UB; ++j) {
             const int ii = i0 + j0 + j;
@@ -844,12 +903,27 @@ __global__ void __launch_bounds__(RPlan<N, PML, BF>::THREADS, 1)
     if constexpr (PL::SPLIT) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(PL::REG_F));
     // ================================================= flux warps
     int fidx = 0;
-    const int sl = flux_slot<SLOTS, PL::EW>(warp, fidx);
+    const int sl = flux_slot<SLOTS, PL::EW, PL::FX>(warp, fidx);
     const uint32_t sA = PL::oA + sl * PL::ASLOT;
     uint64_t* mb = mbar + 12 * sl;
-    const int ft = fidx * 32 + lane;   // flux thread of the slot
-    constexpr int NFT = 32 * PL::FLUXW;
-    constexpr int FT = (T * NF + NFT - 1) / NFT;    // tasks per thread
+    // a lane keeps one face node m, and (where the groups of a slot are a
+    // multiple of 4) one face f: tables and offsets are fixed before the tiles
+    constexpr int FPW = 32 / Nfp;                   // faces a warp takes at once
+    constexpr int FG = FPW * PL::FLUXW;             // face groups of the slot
+    constexpr int FT = (4 * T + FG - 1) / FG;       // faces per thread
+    const int fl = lane / Nfp, m = lane - fl * Nfp;
+    const bool flive = fl < FPW;
+    constexpr int UF = 2;                           // faces in flight in the flux
+    const int grp = fidx * FPW + fl;
+    auto face_of = [&](int u, int& e, int& f) {
+      if constexpr (FG % 4 == 0) {
+        e = (grp >> 2) + u * (FG / 4);
+        f = grp & 3;
+      } else {
+        e = (grp + u * FG) >> 2;
+        f = (grp + u * FG) & 3;
+      }
+    };
     // neighbour traces of a tile (global memory), loaded one tile ahead; the
     // tile's neighbour and code tables come from its early buffer
     float Ep[FT][3], Hp[FT][3], ZPv[FT];
@@ -865,25 +939,34 @@ __global__ void __launch_bounds__(RPlan<N, PML, BF>::THREADS, 1)
         nbs = reinterpret_cast<const int*>(staged(ebuf(sl, itn) + PL::oENB, nbs));
         cds = staged(ebuf(sl, itn) + PL::oECD, cds);
       }
+      // each level of the look-up for all faces before the next one's
+      int nb[FT], np2[FT];
 #pragma unroll
       for (int u = 0; u < FT; ++u) {
-        const int task = ft + u * NFT;
+        int e, f;
+        face_of(u, e, f);
+        const bool on = flive && e < t.ne;
+        nb[u] = on ? nbs[e * 4 + f] : -1;
+        np2[u] = on ? cds[e * 4 + f] : 0;
+      }
+#pragma unroll
+      for (int u = 0; u < FT; ++u) {
+        int e, f;
+        face_of(u, e, f);
+        if (!WADG_INDEX_OK(nb[u] < P.strideQ / (6 * Np) && np2[u] < 24, P.err)) nb[u] = -1;
+        else np2[u] = fperm[(f * 24 + np2[u]) * Nfp + m];
+        if (!WADG_INDEX_OK(np2[u] < Np, P.err)) nb[u] = -1;
+      }
+#pragma unroll
+      for (int u = 0; u < FT; ++u) {
         ZPv[u] = -1.f;
 #pragma unroll
         for (int cc = 0; cc < 3; ++cc) { Ep[u][cc] = 0.f; Hp[u][cc] = 0.f; }
-        if (task < t.ne * NF) {
-          const int e = task / NF, fm = task - e * NF, f = fm / Nfp, m = fm - f * Nfp;
-          const int nb = nbs[e * 4 + f];
-          if (nb >= 0) {
-            const int code = cds[e * 4 + f];
-            if (!WADG_INDEX_OK(nb < P.strideQ / (6 * Np) && code < 24, P.err)) continue;
-            const int np2 = fperm[(f * 24 + code) * Nfp + m];
-            if (!WADG_INDEX_OK(np2 < Np, P.err)) continue;
-            const float* qn = qin + (int64_t)nb * 6 * Np + np2;
+        if (nb[u] >= 0) {
+          const float* qn = qin + (int64_t)nb[u] * 6 * Np + np2[u];
 #pragma unroll
-            for (int cc = 0; cc < 3; ++cc) { Ep[u][cc] = qn[cc * Np]; Hp[u][cc] = qn[(3 + cc) * Np]; }
-            ZPv[u] = P.mat[nb * 3 + 2];
-          }
+          for (int cc = 0; cc < 3; ++cc) { Ep[u][cc] = qn[cc * Np]; Hp[u][cc] = qn[(3 + cc) * Np]; }
+          ZPv[u] = P.mat[nb[u] * 3 + 2];
         }
       }
       return true;
@@ -905,49 +988,66 @@ __global__ void __launch_bounds__(RPlan<N, PML, BF>::THREADS, 1)
       const float* fn_s = reinterpret_cast<const float*>(staged(eb + PL::oEFN, P.fnrm + t.eg0 * 16));
       const float* mat_s = reinterpret_cast<const float*>(staged(eb + PL::oEMAT, P.mat + t.eg0 * 3));
       const float al = (float)P.alpha;
+      // UF faces at a time, their values loaded before any is stored (a face
+      // past the tile's computes on its first element and stores nothing)
 #pragma unroll
-      for (int u = 0; u < FT; ++u) {
-        const int task = ft + u * NFT;
-        if (task >= t.ne * NF) continue;
-        const int e = task / NF, fm = task - e * NF, f = fm / Nfp;
-        const int ni = Fmask[fm];
-        const float* nn = fn_s + e * 16 + f * 4;
-        const float nx = nn[0], ny = nn[1], nz = nn[2], fsc = nn[3];
-        const float* sq = SQ + e * 6 * Np + ni;
-        float Em[3], Hm[3], Eo[3], Ho[3];
+      for (int u0 = 0; u0 < FT; u0 += UF) {
+        float Em_[UF][3], Hm_[UF][3], ZM_[UF];
+        float4 nn_[UF];
 #pragma unroll
-        for (int cc = 0; cc < 3; ++cc) { Em[cc] = sq[cc * Np]; Hm[cc] = sq[(3 + cc) * Np]; }
-        const float ZM = mat_s[e * 3 + 2];
-        float ZP = ZPv[u];
-        if (ZP < 0.f) {   // perfect electric conductor: mirror state
-          ZP = ZM;
+        for (int v = 0; v < UF; ++v) {
+          int e, f;
+          face_of(u0 + v, e, f);
+          if (u0 + v >= FT || e >= t.ne) e = 0;
+          const float* sq = SQ + e * 6 * Np + Fmask[f * Nfp + m];
+          nn_[v] = *reinterpret_cast<const float4*>(fn_s + e * 16 + f * 4);
 #pragma unroll
-          for (int cc = 0; cc < 3; ++cc) { Eo[cc] = -Em[cc]; Ho[cc] = Hm[cc]; }
-        } else {
-#pragma unroll
-          for (int cc = 0; cc < 3; ++cc) { Eo[cc] = Ep[u][cc]; Ho[cc] = Hp[u][cc]; }
+          for (int cc = 0; cc < 3; ++cc) { Em_[v][cc] = sq[cc * Np]; Hm_[v][cc] = sq[(3 + cc) * Np]; }
+          ZM_[v] = mat_s[e * 3 + 2];
         }
-        const float dEx = Eo[0] - Em[0], dEy = Eo[1] - Em[1], dEz = Eo[2] - Em[2];
-        const float dHx = Ho[0] - Hm[0], dHy = Ho[1] - Hm[1], dHz = Ho[2] - Hm[2];
-        const float ndE = nx * dEx + ny * dEy + nz * dEz;
-        const float ndH = nx * dHx + ny * dHy + nz * dHz;
-        const float cHx = ny * dHz - nz * dHy, cHy = nz * dHx - nx * dHz, cHz = nx * dHy - ny * dHx;
-        const float cEx = ny * dEz - nz * dEy, cEy = nz * dEx - nx * dEz, cEz = nx * dEy - ny * dEx;
-        const float YM = __fdividef(1.f, ZM), YP = __fdividef(1.f, ZP);
-        const float sH = __fdividef(fsc, ZM + ZP), sE = __fdividef(fsc, YM + YP);
-        float fo[6];
-        fo[0] = sH * (ZP * cHx - al * (nx * ndE - dEx));
-        fo[1] = sH * (ZP * cHy - al * (ny * ndE - dEy));
-        fo[2] = sH * (ZP * cHz - al * (nz * ndE - dEz));
-        fo[3] = sE * (YP * cEx + al * (nx * ndH - dHx));
-        fo[4] = sE * (YP * cEy + al * (ny * ndH - dHy));
-        fo[5] = sE * (YP * cEz + al * (nz * ndH - dHz));
-        const uint32_t o = cofs<BF>(8 * e, fm, PL::SBLA, PL::LBA);
 #pragma unroll
-        for (int cc = 0; cc < 6; ++cc) {
-          unsigned char* dst = smem + sA + PL::oAL + o + 16 * cc;
-          if constexpr (BF) *reinterpret_cast<__nv_bfloat16*>(dst) = __float2bfloat16_rn(fo[cc]);
-          else *reinterpret_cast<float*>(dst) = to_tf32_int(fo[cc]);
+        for (int v = 0; v < UF; ++v) {
+          const int u = u0 + v;
+          if (u >= FT) break;
+          int e, f;
+          face_of(u, e, f);
+          const int fm = f * Nfp + m;
+          const float nx = nn_[v].x, ny = nn_[v].y, nz = nn_[v].z, fsc = nn_[v].w;
+          const float *Em = Em_[v], *Hm = Hm_[v];
+          float Eo[3], Ho[3];
+          const float ZM = ZM_[v];
+          float ZP = ZPv[u];
+          if (ZP < 0.f) {   // perfect electric conductor: mirror state
+            ZP = ZM;
+#pragma unroll
+            for (int cc = 0; cc < 3; ++cc) { Eo[cc] = -Em[cc]; Ho[cc] = Hm[cc]; }
+          } else {
+#pragma unroll
+            for (int cc = 0; cc < 3; ++cc) { Eo[cc] = Ep[u][cc]; Ho[cc] = Hp[u][cc]; }
+          }
+          const float dEx = Eo[0] - Em[0], dEy = Eo[1] - Em[1], dEz = Eo[2] - Em[2];
+          const float dHx = Ho[0] - Hm[0], dHy = Ho[1] - Hm[1], dHz = Ho[2] - Hm[2];
+          const float ndE = nx * dEx + ny * dEy + nz * dEz;
+          const float ndH = nx * dHx + ny * dHy + nz * dHz;
+          const float cHx = ny * dHz - nz * dHy, cHy = nz * dHx - nx * dHz, cHz = nx * dHy - ny * dHx;
+          const float cEx = ny * dEz - nz * dEy, cEy = nz * dEx - nx * dEz, cEz = nx * dEy - ny * dEx;
+          const float YM = __fdividef(1.f, ZM), YP = __fdividef(1.f, ZP);
+          const float sH = __fdividef(fsc, ZM + ZP), sE = __fdividef(fsc, YM + YP);
+          float fo[6];
+          fo[0] = sH * (ZP * cHx - al * (nx * ndE - dEx));
+          fo[1] = sH * (ZP * cHy - al * (ny * ndE - dEy));
+          fo[2] = sH * (ZP * cHz - al * (nz * ndE - dEz));
+          fo[3] = sE * (YP * cEx + al * (nx * ndH - dHx));
+          fo[4] = sE * (YP * cEy + al * (ny * ndH - dHy));
+          fo[5] = sE * (YP * cEz + al * (nz * ndH - dHz));
+          const uint32_t o = cofs<BF>(8 * e, fm, PL::SBLA, PL::LBA);
+          if (flive && e < t.ne)
+#pragma unroll
+          for (int cc = 0; cc < 6; ++cc) {
+            unsigned char* dst = smem + sA + PL::oAL + o + 16 * cc;
+            if constexpr (BF) *reinterpret_cast<__nv_bfloat16*>(dst) = __float2bfloat16_rn(fo[cc]);
+            else *reinterpret_cast<float*>(dst) = to_tf32_int(fo[cc]);
+          }
         }
       }
       fence_async_smem();
@@ -974,11 +1074,9 @@ cudaError_t rows_configure() {
   // split: refuse a build whose compiled register count would leave it short
   if constexpr (PL::SPLIT) {
     cudaFuncAttributes fa{};
-    cudaError_t e = cudaFuncGetAttributes(&fa, tc_rows_kernel<N, PML, BF>);
+    const cudaError_t e = cudaFuncGetAttributes(&fa, tc_rows_kernel<N, PML, BF>);
     if (e != cudaSuccess) return e;
-    if ((long)fa.numRegs * PL::THREADS <
-        32L * (PL::EW * PL::REG_E + 4 * PL::REG_F + 4 * PL::REG_C))
-      return cudaErrorInvalidConfiguration;
+    if (fa.numRegs < PL::LAUNCH_REGS) return cudaErrorInvalidConfiguration;
   }
   return cudaFuncSetAttribute(tc_rows_kernel<N, PML, BF>,
                               cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1006,46 +1104,53 @@ cudaError_t rows_launch(const StageParams<float>& P, int nb, cudaStream_t s) {
 
 }  // namespace tc
 
-template <bool BF>
+template <bool PML, bool BF>
 cudaError_t configure_rows(int N) {
   switch (N) {
-    case 1: return tc::rows_configure<1, true, BF>();
-    case 2: return tc::rows_configure<2, true, BF>();
-    case 3: return tc::rows_configure<3, true, BF>();
-    case 4: return tc::rows_configure<4, true, BF>();
-    case 5: return tc::rows_configure<5, true, BF>();
+    case 1: return tc::rows_configure<1, PML, BF>();
+    case 2: return tc::rows_configure<2, PML, BF>();
+    case 3: return tc::rows_configure<3, PML, BF>();
+    case 4: return tc::rows_configure<4, PML, BF>();
+    case 5: return tc::rows_configure<5, PML, BF>();
     default: return cudaErrorInvalidValue;
   }
 }
 
 cudaError_t configure_tc_rows(int N, bool bf16) {
-  return bf16 ? configure_rows<true>(N) : configure_rows<false>(N);
+  const cudaError_t e = bf16 ? configure_rows<false, true>(N) : configure_rows<false, false>(N);
+  if (e != cudaSuccess) return e;
+  return bf16 ? configure_rows<true, true>(N) : configure_rows<true, false>(N);
 }
 
-template <bool BF>
+template <bool PML, bool BF>
 cudaError_t launch_rows(int N, const StageParams<float>& P, int nb, cudaStream_t s) {
   switch (N) {
-    case 1: return tc::rows_launch<1, true, BF>(P, nb, s);
-    case 2: return tc::rows_launch<2, true, BF>(P, nb, s);
-    case 3: return tc::rows_launch<3, true, BF>(P, nb, s);
-    case 4: return tc::rows_launch<4, true, BF>(P, nb, s);
-    case 5: return tc::rows_launch<5, true, BF>(P, nb, s);
+    case 1: return tc::rows_launch<1, PML, BF>(P, nb, s);
+    case 2: return tc::rows_launch<2, PML, BF>(P, nb, s);
+    case 3: return tc::rows_launch<3, PML, BF>(P, nb, s);
+    case 4: return tc::rows_launch<4, PML, BF>(P, nb, s);
+    case 5: return tc::rows_launch<5, PML, BF>(P, nb, s);
     default: return cudaErrorInvalidValue;
   }
 }
 
-cudaError_t launch_pml_tc_rows(int N, const StageParams<float>& P, int nb, cudaStream_t s,
-                               bool bf16) {
+cudaError_t launch_tc_rows(int N, bool pml, const StageParams<float>& P, int nb, cudaStream_t s,
+                           bool bf16) {
   // the bulk copies move whole 16-byte covers of each block: the arrays must
   // start on 16-byte boundaries (cudaMalloc gives 256)
   const uintptr_t a =
       reinterpret_cast<uintptr_t>(P.qin) | reinterpret_cast<uintptr_t>(P.qout) |
-      reinterpret_cast<uintptr_t>(P.resq) | reinterpret_cast<uintptr_t>(P.p) |
-      reinterpret_cast<uintptr_t>(P.resp) | reinterpret_cast<uintptr_t>(P.sig) |
+      reinterpret_cast<uintptr_t>(P.resq) | reinterpret_cast<uintptr_t>(P.nbr) |
+      reinterpret_cast<uintptr_t>(P.code) |
+      (pml ? reinterpret_cast<uintptr_t>(P.p) | reinterpret_cast<uintptr_t>(P.resp) |
+                 reinterpret_cast<uintptr_t>(P.sig)
+           : 0) |
       reinterpret_cast<uintptr_t>(P.fnrm) | reinterpret_cast<uintptr_t>(P.geof) |
       reinterpret_cast<uintptr_t>(P.mat);
   if (a & 15) return cudaErrorMisalignedAddress;
-  return bf16 ? launch_rows<true>(N, P, nb, s) : launch_rows<false>(N, P, nb, s);
+  if (pml)
+    return bf16 ? launch_rows<true, true>(N, P, nb, s) : launch_rows<true, false>(N, P, nb, s);
+  return bf16 ? launch_rows<false, true>(N, P, nb, s) : launch_rows<false, false>(N, P, nb, s);
 }
 
 }  // namespace wadg
