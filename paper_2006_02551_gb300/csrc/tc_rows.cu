@@ -74,8 +74,9 @@ struct RPlan {
   static constexpr int NqP = (Nq + 3) & ~3;         // stride of the sigma samples
   // ... and of a staged row of them: the lanes of an element read three rows at
   // once, which must not start on the same banks (a multiple of 16 floats would
-  // put rows 0 and 2 there; such rows are copied one by one)
-  static constexpr int SGR = NqP % 16 == 0 ? NqP + 4 : NqP;
+  // put rows 0 and 2 there; such rows are copied one by one, except at N = 2, where
+  // 24 copies of 64 bytes cost more than the conflict: 79.5 against 64.3 us)
+  static constexpr int SGR = NqP % 16 == 0 && NqP > 16 ? NqP + 4 : NqP;
   static constexpr int CW = O::CW, KS = O::KS;
   __host__ __device__ static constexpr int rupK(int x) { return (x + KS - 1) / KS * KS; }
   static constexpr int NpK = rupK(Np), NFK = rupK(NF), NqK = rupK(Nq);
