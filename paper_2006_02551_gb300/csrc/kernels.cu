@@ -6,31 +6,31 @@
 
 namespace wadg {
 
-template <typename Real, int N, bool PML, bool KAPPA, bool STORED = false, int QC = 0>
-__global__ void __launch_bounds__(Tile<Real, N, PML, 0, QC>::THREADS)
+template <typename Real, int N, bool KAPPA, bool STORED = false, int QC = 0>
+__global__ void __launch_bounds__(Tile<Real, N, QC>::THREADS)
 stage_kernel(const StageParams<Real> P) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  stage_body<Real, N, PML, KAPPA, STORED, 0, QC>(P, smem_raw, blockIdx.x, gridDim.x);
+  stage_body<Real, N, KAPPA, STORED, QC>(P, smem_raw, blockIdx.x, gridDim.x);
 }
 
-template <typename Real, int N, bool PML, bool KAPPA, bool STORED = false, int QC = 0>
+template <typename Real, int N, bool KAPPA, bool STORED = false, int QC = 0>
 static cudaError_t configure_one() {
-  using TL = Tile<Real, N, PML, 0, QC>;
-  return cudaFuncSetAttribute(stage_kernel<Real, N, PML, KAPPA, STORED, QC>,
+  using TL = Tile<Real, N, QC>;
+  return cudaFuncSetAttribute(stage_kernel<Real, N, KAPPA, STORED, QC>,
                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TL::smem);
 }
 
 // resident blocks per SM of one stage-kernel instance (cached per instance)
-template <typename Real, int N, bool PML, bool KAPPA, bool STORED = false, int QC = 0>
+template <typename Real, int N, bool KAPPA, bool STORED = false, int QC = 0>
 static int resident_blocks() {
   static int cached = 0;
   if (cached == 0) {
-    using TL = Tile<Real, N, PML, 0, QC>;
+    using TL = Tile<Real, N, QC>;
     int nb = 0, dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &nb, stage_kernel<Real, N, PML, KAPPA, STORED, QC>, TL::THREADS, TL::smem) !=
+            &nb, stage_kernel<Real, N, KAPPA, STORED, QC>, TL::THREADS, TL::smem) !=
             cudaSuccess ||
         nb < 1)
       nb = 1;
@@ -39,25 +39,25 @@ static int resident_blocks() {
   return cached;
 }
 
-template <typename Real, int N, bool PML, bool KAPPA, bool STORED = false, int QC = 0>
+template <typename Real, int N, bool KAPPA, bool STORED = false, int QC = 0>
 static cudaError_t launch_one(const StageParams<Real>& P, int nb, cudaStream_t s) {
-  using TL = Tile<Real, N, PML, 0, QC>;
+  using TL = Tile<Real, N, QC>;
   if (P.n_elem <= 0) return cudaSuccess;
   StageParams<Real> Q = P;
   Q.nb = nb;
   const long long tiles = (long long)((P.n_elem + TL::T - 1) / TL::T) * nb;
   const int grid =
-      (int)std::min<long long>(tiles, resident_blocks<Real, N, PML, KAPPA, STORED, QC>());
-  stage_kernel<Real, N, PML, KAPPA, STORED, QC><<<grid, TL::THREADS, TL::smem, s>>>(Q);
+      (int)std::min<long long>(tiles, resident_blocks<Real, N, KAPPA, STORED, QC>());
+  stage_kernel<Real, N, KAPPA, STORED, QC><<<grid, TL::THREADS, TL::smem, s>>>(Q);
   return cudaGetLastError();
 }
 
 template <typename Real, int N>
 static cudaError_t configure_n() {
-  cudaError_t e = configure_one<Real, N, true, false>();
-  if (e == cudaSuccess) e = configure_one<Real, N, true, true>();
-  if (e == cudaSuccess) e = configure_one<Real, N, true, false, false, 1>();
-  if (e == cudaSuccess) e = configure_one<Real, N, true, true, false, 1>();
+  cudaError_t e = configure_one<Real, N, false>();
+  if (e == cudaSuccess) e = configure_one<Real, N, true>();
+  if (e == cudaSuccess) e = configure_one<Real, N, false, false, 1>();
+  if (e == cudaSuccess) e = configure_one<Real, N, true, false, 1>();
   return e;
 }
 
@@ -79,11 +79,11 @@ template <typename Real, int N>
 static cudaError_t dispatch_pml(bool kappa, const StageParams<Real>& P, int nb, cudaStream_t s,
                                 int qc) {
   if (qc) {
-    if (kappa) return launch_one<Real, N, true, true, false, 1>(P, nb, s);
-    return launch_one<Real, N, true, false, false, 1>(P, nb, s);
+    if (kappa) return launch_one<Real, N, true, false, 1>(P, nb, s);
+    return launch_one<Real, N, false, false, 1>(P, nb, s);
   }
-  if (kappa) return launch_one<Real, N, true, true>(P, nb, s);
-  return launch_one<Real, N, true, false>(P, nb, s);
+  if (kappa) return launch_one<Real, N, true>(P, nb, s);
+  return launch_one<Real, N, false>(P, nb, s);
 }
 
 template <typename Real>
@@ -106,8 +106,8 @@ template cudaError_t launch_stage<float>(int, bool, const StageParams<float>&, i
 // ------------------------------------------------------- stored-matrix scheme
 template <typename Real, int N>
 static cudaError_t configure_stored_n() {
-  cudaError_t e = configure_one<Real, N, true, false, true>();
-  if (e == cudaSuccess) e = configure_one<Real, N, true, true, true>();
+  cudaError_t e = configure_one<Real, N, false, true>();
+  if (e == cudaSuccess) e = configure_one<Real, N, true, true>();
   return e;
 }
 
@@ -127,8 +127,8 @@ template cudaError_t configure_stored_kernels<float>(int);
 
 template <typename Real, int N>
 static cudaError_t launch_stored_n(bool kappa, const StageParams<Real>& P, int nb, cudaStream_t s) {
-  return kappa ? launch_one<Real, N, true, true, true>(P, nb, s)
-               : launch_one<Real, N, true, false, true>(P, nb, s);
+  return kappa ? launch_one<Real, N, true, true>(P, nb, s)
+               : launch_one<Real, N, false, true>(P, nb, s);
 }
 
 template <typename Real>

@@ -1,5 +1,6 @@
-// Body of the CUDA-core DGTD stage (shared by the per-class launches in
-// kernels.cu and the grouped launch in group.cu): one pass over a tile of
+// Body of the dense CUDA-core DGTD stage (kernels.cu): the PML class with a
+// volume rule without symmetry, and with the stored-matrix scheme; everything
+// else runs the symmetric stage (sym_body.cuh).  One pass over a tile of
 // elements computes the right-hand side of the semi-discrete system and
 // applies the low-storage Runge-Kutta update.
 //
@@ -7,7 +8,7 @@
 //   * face traces through the neighbour map and the upwind flux,
 //   * volume curl through the reference differentiation matrices and the
 //     metric terms, LIFT of the scaled flux (curl operator Cbar_k),
-//   * in PML elements the weight-adjusted terms of eqs. 26-29: interpolate
+//   * the weight-adjusted terms of eqs. 26-29: interpolate
 //     E, H, P^E, P^H to the quadrature nodes (V_q), form the CPML tensors of
 //     eq. 9 pointwise from the stored sigma_u (kappa_u) samples, project
 //     back (P_q); with kappa = 1 the outer P_q a^{-1} V_q is the identity
@@ -38,29 +39,27 @@ struct Dims {
 
 // Launch configuration: persistent blocks, the reference operators staged in
 // shared memory once per block, tiles of T elements processed in a loop.
-template <typename Real, int N, bool PML, int NT_ = 0, int QC = 0>
+template <typename Real, int N, int QC = 0>
 struct Tile {
   using D = Dims<N, QC>;
-  // threads of a block: the single-class launches use 512 for FP32 PML tiles;
-  // the grouped launch fixes 256 for every class
-  static constexpr int THREADS = NT_ > 0 ? NT_ : ((sizeof(Real) == 4 && PML) ? 512 : 256);
-  static constexpr int CF = PML ? 12 : 6;                  // field components held
+  static constexpr int THREADS = sizeof(Real) == 4 ? 512 : 256;
+  static constexpr int CF = 12;                            // field components held
   static constexpr int f_sz = D::Np * CF;                  // F[e][j][CF]
-  static constexpr int u_sz = PML ? ((D::NF * 6 > D::NqP * 12) ? D::NF * 6 : D::NqP * 12)
-                                  : D::NF * 6;             // flux[e][f][6] / tz[e][q][12]
-  static constexpr int r_sz = PML ? D::NpP * 6 : 0;        // rs[e][i][6]
+  static constexpr int u_sz = D::NF * 6 > D::NqP * 12 ? D::NF * 6
+                                                         : D::NqP * 12;   // flux[e][f][6] / tz[e][q][12]
+  static constexpr int r_sz = D::NpP * 6;                  // rs[e][i][6]
   static constexpr int per_elem = f_sz + u_sz + r_sz + 16 + 12;
-  // operators: DrT DsT DtT [Np][NpP], LIFTT [NF][NpP] (+ VqT [Np][NqP], PqT [Nq][NpP]);
+  // operators: DrT DsT DtT [Np][NpP], LIFTT [NF][NpP], VqT [Np][NqP], PqT [Nq][NpP];
   // staged in shared memory when they fit, read through L1 otherwise
   static constexpr int ops_all = 3 * D::Np * D::NpP + D::NF * D::NpP +
-                                 (PML ? D::Np * D::NqP + D::Nq * D::NpP : 0);
+                                 D::Np * D::NqP + D::Nq * D::NpP;
   static constexpr bool OPS_SMEM = ops_all * (int)sizeof(Real) <= 160 * 1024;
   static constexpr int ops_sz = OPS_SMEM ? ops_all : 0;
-  static constexpr int budget = (PML || sizeof(Real) == 8) ? 200 * 1024 : 100 * 1024;
+  static constexpr int budget = 200 * 1024;
   static constexpr int avail = budget - ops_sz * (int)sizeof(Real) - 256;
   static constexpr int t0 = avail / (per_elem * (int)sizeof(Real));
   // enough tiles of work per phase for the block's threads, not more
-  static constexpr int t_tasks = PML ? THREADS / D::NQQ : THREADS / (2 * D::NIQ);
+  static constexpr int t_tasks = THREADS / D::NQQ;
   static constexpr int t1 = t0 < t_tasks ? t0 : t_tasks;
   static constexpr int T = t1 < 1 ? 1 : (t1 > 32 ? 32 : t1);
   static constexpr size_t smem =
@@ -117,27 +116,23 @@ __device__ __forceinline__ void lds2(const double* p, double* v) {
 
 // Stage kernel.  Threads work on register tiles: 4 nodes x 3 components x 3
 // reference derivatives (curl), 4 quadrature points x 12 components (V_q),
-// 4 nodes x 4 components (P_q).  All operator reads come from shared memory.
-// Body of the stage kernel for one element class of one context; smem_raw is
-// the block's dynamic shared memory.  Static schedule: block `bid` of `nblk`
-// takes tiles bid, bid + nblk, ...  Dynamic schedule (dyn != nullptr, the
-// grouped launch): the block takes tiles from the counter *dyn until they run
-// out.
-template <typename Real, int N, bool PML, bool KAPPA, bool STORED, int NT_, int QC = 0>
+// smem_raw is the block's dynamic shared memory; block `bid` of `nblk` takes
+// tiles bid, bid + nblk, ...
+template <typename Real, int N, bool KAPPA, bool STORED, int QC = 0>
 __device__ __forceinline__ void stage_body(const StageParams<Real>& P, unsigned char* smem_raw,
-                                           int bid, int nblk, int* dyn = nullptr) {
+                                           int bid, int nblk) {
   using D = Dims<N, QC>;
   constexpr int Np = D::Np, Nfp = D::Nfp, Nq = D::Nq, NF = D::NF;
   constexpr int NpP = D::NpP, NqP = D::NqP, NIQ = D::NIQ, NQQ = D::NQQ;
-  using TL = Tile<Real, N, PML, NT_, QC>;
+  using TL = Tile<Real, N, QC>;
   constexpr int T = TL::T, CF = TL::CF, NT = TL::THREADS;
   Real* sm = reinterpret_cast<Real*>(smem_raw);
   const Real* DrT = TL::OPS_SMEM ? sm : P.ops;   // operators
   const Real* DsT = DrT + Np * NpP;
   const Real* DtT = DsT + Np * NpP;
   const Real* LIFTT = DtT + Np * NpP;
-  const Real* VqT = LIFTT + NF * NpP;   // PML only
-  const Real* PqT = VqT + Np * NqP;     // PML only
+  const Real* VqT = LIFTT + NF * NpP;
+  const Real* PqT = VqT + Np * NqP;  
   // elements per tile: T, or fewer when the launch asks for smaller tiles
   // (the shared-memory carve-up follows, so smaller tiles need less of it)
   const int TE = P.tile_elems > 0 && P.tile_elems < T ? P.tile_elems : T;
@@ -167,24 +162,7 @@ __device__ __forceinline__ void stage_body(const StageParams<Real>& P, unsigned 
   const int tiles_per_batch = (P.n_elem + TE - 1) / TE;
   const int ntiles = tiles_per_batch * P.nb;
 
-  // dynamic schedule: thread 0 claims the next tile at the start of the
-  // current one and publishes it at the end, so the atomic's round trip
-  // overlaps the tile's work (a claim past the last tile is left unused)
-  __shared__ int dyn_tile;
-  int claimed = 0;
-  auto claim = [&]() {
-    if (dyn && tid == 0) claimed = atomicAdd(dyn, 1);
-  };
-  auto next_tile = [&](int cur) -> int {
-    if (!dyn) return cur < 0 ? bid : cur + nblk;
-    __syncthreads();   // every thread has read the previous value
-    if (tid == 0) dyn_tile = claimed;
-    __syncthreads();
-    return dyn_tile;
-  };
-  claim();
-  for (int tile = next_tile(-1); tile < ntiles; tile = next_tile(tile)) {
-  claim();
+  for (int tile = bid; tile < ntiles; tile += nblk) {
   const int b = tile / tiles_per_batch;
   const int t0 = (tile - b * tiles_per_batch) * TE;
   const int ne = min(TE, P.n_elem - t0);
@@ -204,12 +182,10 @@ __device__ __forceinline__ void stage_body(const StageParams<Real>& P, unsigned 
     const int e = idx / (6 * Np), r = idx - e * 6 * Np, c = r / Np, j = r - c * Np;
     F[(e * Np + j) * CF + c] = qin[(int64_t)eg0 * 6 * Np + idx];
   }
-  if (PML) {
-    const Real* pin = pio + (int64_t)ep0 * 6 * Np;
-    for (int idx = tid; idx < ne * 6 * Np; idx += NT) {
-      const int e = idx / (6 * Np), r = idx - e * 6 * Np, c = r / Np, j = r - c * Np;
-      F[(e * Np + j) * CF + 6 + c] = pin[idx];
-    }
+  const Real* pin = pio + (int64_t)ep0 * 6 * Np;
+  for (int idx = tid; idx < ne * 6 * Np; idx += NT) {
+    const int e = idx / (6 * Np), r = idx - e * 6 * Np, c = r / Np, j = r - c * Np;
+    F[(e * Np + j) * CF + 6 + c] = pin[idx];
   }
   for (int idx = tid; idx < ne * 16; idx += NT)
     nrm[idx] = P.fnrm[(int64_t)eg0 * 16 + idx];   // n_x, n_y, n_z, Fscale per face
@@ -276,11 +252,11 @@ __device__ __forceinline__ void stage_body(const StageParams<Real>& P, unsigned 
   __syncthreads();
   const int nsrc_l = min(nsl, 64);
 
-  // ---- phase 2 (+ phase 3 in PML tiles, same loop: they are independent)
+  // ---- phases 2 and 3
   //   curl task (e, fld, iq): fld 0: Cbar(E) -> rhs_H = -Cbar(E)/mu,
   //                           fld 1: Cbar(H) -> rhs_E =  Cbar(H)/eps
   //   V_q task (e, qq): 12 fields at 4 quadrature points, then eq. 9 pointwise
-  // In PML tiles the V_q results go to TZ, which aliases FL; so the V_q tasks
+  // The V_q results go to TZ, which aliases FL; so the V_q tasks
   // must not start before every curl task has read FL: they run after a
   // barrier in the second loop below.
   const int n2 = ne * 2 * NIQ;
@@ -366,27 +342,12 @@ __device__ __forceinline__ void stage_body(const StageParams<Real>& P, unsigned 
         for (int n = 0; n < 4; ++n) out[c][n] *= ie;
     }
     const int oc = fld == 0 ? 3 : 0;   // rhs_H lands on components 3..5
-    if (!PML) {
 #pragma unroll
-      for (int c = 0; c < 3; ++c)
+    for (int c = 0; c < 3; ++c)
 #pragma unroll
-        for (int n = 0; n < 4; ++n) {
-          const int i = 4 * iq + n;
-          if (i < Np) {
-            const int64_t gi = ((int64_t)eg * 6 + oc + c) * Np + i;
-            const Real rr = rka * resq[gi] + rdt * out[c][n];
-            resq[gi] = rr;
-            qout[gi] = F[(e * Np + i) * CF + oc + c] + rkb * rr;
-          }
-        }
-    } else {
-#pragma unroll
-      for (int c = 0; c < 3; ++c)
-#pragma unroll
-        for (int n = 0; n < 4; ++n) RS[(e * NpP + 4 * iq + n) * 6 + oc + c] = out[c][n];
-    }
+      for (int n = 0; n < 4; ++n) RS[(e * NpP + 4 * iq + n) * 6 + oc + c] = out[c][n];
   }
-  if (PML && STORED) {
+  if (STORED) {
   __syncthreads();   // RS complete
 
   // ---- stored-matrix scheme (eqs. 10-13): per axis u, 4 nodes per task,
@@ -492,7 +453,7 @@ __device__ __forceinline__ void stage_body(const StageParams<Real>& P, unsigned 
   }
   }  // KAPPA
   }  // stored
-  if (PML && !STORED) {
+  if (!STORED) {
   __syncthreads();   // FL is reused as TZ below
 
   // ---- phase 3: V_q of the 12 fields at 4 quadrature points; eq. 9 pointwise
@@ -677,7 +638,7 @@ __device__ __forceinline__ void stage_body(const StageParams<Real>& P, unsigned 
     }
   }
   }  // KAPPA
-  }  // PML
+  }  // weight-adjusted
   }  // tile loop
 }
 

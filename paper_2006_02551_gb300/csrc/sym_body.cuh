@@ -27,7 +27,8 @@
 //            memory order
 // Reference coefficients are the same for all lanes of a warp (rows are the
 // lanes): one broadcast load each in FP64; in FP32, where those loads were the
-// bound, constant-bank operands.
+// bound, constant-bank operands for V_q and P_q (N <= 4) and, at N <= 2, for the
+// derivative and LIFT blocks.
 //
 // What bounds it now: FP64 the FP64 pipe; FP32 the barriers between phases of
 // unequal warps, instruction fetch and shared-memory loads (issue slots 42 %
@@ -36,7 +37,8 @@
 // Measured, a step against the dense stage: FP32, 384,000 tets, N = 4, compact
 // rule: 17.6 -> 4.7 ms; FP32, 162,000 tets, N = 3, 16 excitations: 59 -> 18.5
 // ms; FP64, 48,000 tets, N = 4: 33.3 -> 12.5 ms; FP64, 384 tets, N = 3, (N+1)^3
-// rule: 1.16 -> 0.28 ms (mostly the smaller tiles); kappa = 2, 29,478 tets, N =
+// rule: 1.16 -> 0.21 ms (mostly the smaller tiles, then
+// sym_both_kernel); kappa = 2, 29,478 tets, N =
 // 4: 1.78 -> 0.74 ms.  Of the FP32 step, the first version (scalar
 // multiplications, face factors computed in the kernel, the update's registers
 // loaded one by one) took 5.9 ms; the update's loads were 9,500 of a PML tile's
@@ -56,34 +58,26 @@
 
 namespace wadg {
 
-
-// FP32 derivative and LIFT blocks (they depend on the order alone) in constant
-// memory: a warp's coefficient comes through the constant cache to the uniform
-// registers, where a broadcast from shared memory takes a cycle of the SM's
-// load path per coefficient (the curl was bound by those).  One copy per
-// translation unit, written by upload_sym_constants.
-static __constant__ float c_sym1[SymLayout<1>::oV], c_sym2[SymLayout<2>::oV],
-    c_sym3[SymLayout<3>::oV], c_sym4[SymLayout<4>::oV], c_sym5[SymLayout<5>::oV];
+// FP32 derivative and LIFT blocks (they depend on the order alone) of N <= 2 in
+// constant memory: a warp's coefficient comes through the constant cache to the
+// uniform registers, where a broadcast from shared memory takes a cycle of the
+// SM's load path per coefficient.  Above N = 2 they miss the constant cache
+// (N = 4: 2.34 against 1.74 ns per non-PML element) and stay in shared memory.
+// One copy per translation unit, written by upload_sym_constants.
+static __constant__ float c_sym1[SymLayout<1>::oV], c_sym2[SymLayout<2>::oV];
 template <int N>
 __device__ __forceinline__ const float* sym_const() {
+  static_assert(N <= 2, "orders in constant memory");
   if constexpr (N == 1) return c_sym1;
-  else if constexpr (N == 2) return c_sym2;
-  else if constexpr (N == 3) return c_sym3;
-  else if constexpr (N == 4) return c_sym4;
-  else return c_sym5;
+  else return c_sym2;
 }
 // this translation unit's copy for order N on the current device (the same
 // bytes whenever it is written)
 inline cudaError_t upload_sym_constants(int N) {
+  if (N > 2) return cudaSuccess;
   const std::vector<float>& h = sym_constants(N);
   const size_t n = h.size() * sizeof(float);
-  switch (N) {
-    case 1: return cudaMemcpyToSymbol(c_sym1, h.data(), n);
-    case 2: return cudaMemcpyToSymbol(c_sym2, h.data(), n);
-    case 3: return cudaMemcpyToSymbol(c_sym3, h.data(), n);
-    case 4: return cudaMemcpyToSymbol(c_sym4, h.data(), n);
-    default: return cudaMemcpyToSymbol(c_sym5, h.data(), n);
-  }
+  return N == 1 ? cudaMemcpyToSymbol(c_sym1, h.data(), n) : cudaMemcpyToSymbol(c_sym2, h.data(), n);
 }
 
 // V_q and P_q coefficients of a volume rule (n each) as a kernel parameter,
