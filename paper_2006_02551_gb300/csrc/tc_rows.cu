@@ -785,7 +785,7 @@ __global__ void __launch_bounds__(RPlan<N, PML, BF>::THREADS, 1)
           const float a1 = __shfl_sync(0xffffffffu, o1, s1);
           const float a2 = __shfl_sync(0xffffffffu, o2, s2);
           const float cr = a1 - a2 + lf;   // (curl of the partner field) + LIFT term
-          rhs[ic + j] = kc * cr;
+          rhs[ic + j] = PML ? kc * cr : cr;
         }
       };
       constexpr int CB = NHC < 12 ? NHC : 12;   // nodes per batch of loads
@@ -806,8 +806,15 @@ __global__ void __launch_bounds__(RPlan<N, PML, BF>::THREADS, 1)
                            (float)sd.dir[c];
 #pragma unroll
           for (int ic = 0; ic < NHC; ++ic)
-            if (i0 + ic < i1) rhs[ic] -= ie * jt * P.src_w[s * Np + i0 + ic];
+            if (i0 + ic < i1)
+              rhs[ic] -= PML ? ie * jt * P.src_w[s * Np + i0 + ic] : jt * P.src_w[s * Np + i0 + ic];
         }
+      }
+      // the non-PML class scales the curl and the source together, as the
+      // operator-rows kernel did (the same bits in elements with a source)
+      if constexpr (!PML) {
+#pragma unroll
+        for (int ic = 0; ic < NHC; ++ic) rhs[ic] *= kc;
       }
       // the P_q outputs (s for E, H rows; the right-hand side for P rows)
       uint32_t sz[2 * NHC];
