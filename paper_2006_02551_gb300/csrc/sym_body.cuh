@@ -31,8 +31,8 @@
 // derivative and LIFT blocks.
 //
 // What bounds it now: FP64 the FP64 pipe; FP32 the barriers between phases of
-// unequal warps, instruction fetch and shared-memory loads (issue slots 42 %
-// busy, load path 48 %, DRAM 26 %: ncu, PML class, 82,944 tets, N = 4).
+// unequal warps, instruction fetch and shared-memory loads (issue slots 39 %
+// busy, load path 50 %, DRAM 25 %: ncu, PML class, 82,944 tets, N = 4).
 //
 // Measured, a step against the dense stage: FP32, 384,000 tets, N = 4, compact
 // rule: 17.6 -> 4.7 ms; FP32, 162,000 tets, N = 3, 16 excitations: 59 -> 18.5
