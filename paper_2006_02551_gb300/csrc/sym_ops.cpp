@@ -177,34 +177,40 @@ SymRule detect_symmetry(const RefOps& R) {
     lam[4 * q + 3] = 0.5 * (1 + R.tq[q]);
     lam[4 * q] = -0.5 * (1 + R.rq[q] + R.sq[q] + R.tq[q]);
   }
-  // the point at the image of q under the vertex map `im`, -1 if none
-  auto image = [&](int q, const int im[4]) -> int {
-    for (int p = 0; p < n; ++p) {
-      bool same = std::fabs(R.wq[p] - R.wq[q]) <= 1e-13 * std::fabs(R.wq[q]);
-      for (int v = 0; v < 4 && same; ++v)
-        same = std::fabs(lam[4 * p + v] - lam[4 * q + im[v]]) <= 1e-14;
-      if (same) return p;
-    }
-    return -1;
+  // whether point p lies at the image of q under the vertex map `im`
+  auto at_image = [&](int p, int q, const int im[4]) {
+    for (int v = 0; v < 4; ++v)
+      if (!(std::fabs(lam[4 * p + v] - lam[4 * q + im[v]]) <= 1e-14)) return false;
+    return true;
   };
   for (int G : {4, 2}) {
     SymRule S;
     S.G = G;
+    // Every point belongs to exactly one orbit.  Within an orbit a location has
+    // one point (a point that an element fixes, or that two elements reach,
+    // appears for each of them); a point listed twice forms orbits with the
+    // other listings of its images.
     std::vector<char> seen(n, 0);
     bool ok = true;
     for (int q = 0; q < n && ok; ++q) {
       if (seen[q]) continue;
       int sl[4] = {q, q, q, q};
+      seen[q] = 1;
       for (int y = 1; y < G && ok; ++y) {
-        int im[4];
+        int im[4], p = -1;
         for (int v = 0; v < 4; ++v) im[v] = G == 4 ? v4_image(y, v) : (v < 2 ? 1 - v : v);
-        sl[y] = image(q, im);
-        ok = sl[y] >= 0;
+        for (int z = 0; z < y && p < 0; ++z)
+          if (at_image(sl[z], q, im)) p = sl[z];
+        for (int k = 0; k < n && p < 0; ++k)
+          if (!seen[k] && std::fabs(R.wq[k] - R.wq[q]) <= 1e-13 * std::fabs(R.wq[q]) &&
+              at_image(k, q, im))
+            p = k;
+        ok = p >= 0;
+        if (!ok) break;
+        sl[y] = p;
+        seen[p] = 1;
       }
-      for (int y = 0; y < G && ok; ++y) {
-        seen[sl[y]] = 1;
-        S.slots.push_back(sl[y]);
-      }
+      S.slots.insert(S.slots.end(), sl, sl + G);
     }
     if (!ok) continue;
     while (S.slots.size() % 4) S.slots.push_back(-1);
