@@ -600,7 +600,7 @@ wadg_status rebuild_typed(wadg_ctx* ctx) {
     // a CUDA-core context
     const bool groups = !ctx->tc;
     const int ns = groups ? 4 * sample_groups(ctx) : (Nq + 3) & ~3;
-    std::vector<double> rq(3 * (size_t)ns, 2.0);   // 2: padding
+    std::vector<double> rq(3 * (size_t)ns, kPadPoint);
     for (int i = 0; i < ns; ++i) {
       const int q = groups && ctx->sym.G ? ctx->sym.slots[i] : (i < Nq ? i : -1);
       if (q < 0) continue;

@@ -435,7 +435,7 @@ __global__ void pml_samples_kernel(int n, bool groups, int K1, int K0, const dou
   auto at = [&](int u) {
     return (int64_t)e * 3 * n + (groups ? (q >> 2) * 12 + u * 4 + (q & 3) : u * n + q);
   };
-  if (rq[q * 3] > 1.0) {   // padding
+  if (rq[q * 3] == kPadPoint) {
     for (int u = 0; u < 3; ++u) {
       sig[at(u)] = Real(0);
       if (kap) kap[at(u)] = Real(1);

@@ -231,8 +231,10 @@ cudaError_t launch_sym_geometry(int64_t K, const double* geo, const double* vert
                                 const Real* fnrm, const Real* mat, const int* nbr,
                                 const unsigned char* code, Real* facex, Real* geox,
                                 cudaStream_t s);
-// n sample places per element and axis at the reference points rq [n][3] (a
-// coordinate above 1: padding); groups: [group][3][4] blocks of sigma / eps0,
+constexpr double kPadPoint = 4.0;
+// n sample places per element and axis at the reference points rq [n][3]
+// (kPadPoint: padding, a value that no point of a rule has; an accepted point's
+// coordinates reach 1 + 6e-12); groups: [group][3][4] blocks of sigma / eps0,
 // else [3][n] blocks of it
 template <typename Real>
 cudaError_t launch_pml_samples(int n, bool groups, int K1, int K0, const double* verts,
