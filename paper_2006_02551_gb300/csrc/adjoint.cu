@@ -94,7 +94,7 @@ struct AdjTile {
   static constexpr int budget = 80 * 1024;
   static constexpr int t0 = budget / (per * (int)sizeof(Real));
   static constexpr int T = t0 < 1 ? 1 : (t0 > 8 ? 8 : t0);
-  static constexpr size_t smem = (size_t)T * per * sizeof(Real) + 64 * sizeof(int);
+  static constexpr size_t smem = (size_t)T * per * sizeof(Real);
 };
 
 template <typename Real>
@@ -121,8 +121,7 @@ __global__ void __launch_bounds__(kAdjThreads) adj_main_kernel(const AdjParams<R
   Real* ZZ = FLH + T * NF * 3;                     // [T][NqP][12] (PML)
   Real* GE = ZZ + (PML ? T * 12 * NqP : 0);        // [T] dJ/deps_k
   Real* MET = GE + T * 16;                         // [T][9] metric r_x .. t_z
-  int* srcl = reinterpret_cast<int*>(MET + T * 16);
-  __shared__ int nsl;
+  __shared__ int nsl, src0;                        // the tile's sources: count, first
   __shared__ double red[6][kAdjThreads / 32];
 
   constexpr int NFP = (NF + 3) & ~3;
@@ -156,7 +155,10 @@ __global__ void __launch_bounds__(kAdjThreads) adj_main_kernel(const AdjParams<R
   const Real* Gb = A.G + (int64_t)b * A.K * NF * 6;
 
   // ---- load mu, stage input, clear accumulators
-  if (tid == 0) nsl = 0;
+  if (tid == 0) {
+    nsl = 0;
+    src0 = A.nsrc;
+  }
   for (int idx = tid; idx < ne * 6 * Np; idx += kAdjThreads) {
     const int e = idx / (6 * Np), r = idx - e * 6 * Np;
     const int64_t gi = (int64_t)eg0 * 6 * Np + idx;
@@ -182,8 +184,8 @@ __global__ void __launch_bounds__(kAdjThreads) adj_main_kernel(const AdjParams<R
   for (int s = tid; s < A.nsrc; s += kAdjThreads) {
     const SrcDev& sd = A.src[s];
     if (sd.batch == b && sd.elem >= eg0 && sd.elem < eg0 + ne) {
-      const int slot = atomicAdd(&nsl, 1);
-      if (slot < 64) srcl[slot] = s;
+      atomicAdd(&nsl, 1);
+      atomicMin(&src0, s);
     }
   }
 
@@ -292,7 +294,7 @@ __global__ void __launch_bounds__(kAdjThreads) adj_main_kernel(const AdjParams<R
     atomic_add_real(&GE[e], ge);
   }
   __syncthreads();
-  const int nsrc_l = min(nsl, 64);
+  const int sb0 = src0, sb1 = sb0 + nsl;
 
   // ---- volume: curl^T of (mu_E/eps, -mu_H/mu); forward Cbar(H) for dJ/deps
   for (int idx = tid; idx < ne * Np; idx += kAdjThreads) {
@@ -356,13 +358,13 @@ __global__ void __launch_bounds__(kAdjThreads) adj_main_kernel(const AdjParams<R
 #pragma unroll
       for (int c = 0; c < 3; ++c) CH[c] += L * FLH[(e * NF + fm) * 3 + c];
     }
-    for (int s = 0; s < nsrc_l; ++s) {
-      const SrcDev& sd = A.src[srcl[s]];
+    for (int s = sb0; s < sb1; ++s) {
+      const SrcDev& sd = A.src[s];
       if (sd.elem != eg) continue;
       const double tau = sd.width;
       const double g = exp(-(tst - sd.t0) * (tst - sd.t0) / (4.0 * tau * tau));
       const Real jt = (Real)(sd.amp * (-(tst - sd.t0) / (2.0 * tau * tau)) * g);
-      const Real w = A.src_w[srcl[s] * Np + i];
+      const Real w = A.src_w[(int64_t)s * Np + i];
 #pragma unroll
       for (int c = 0; c < 3; ++c) CH[c] -= jt * (Real)sd.dir[c] * w;
     }

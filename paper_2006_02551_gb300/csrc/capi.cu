@@ -664,14 +664,29 @@ wadg_status upload_sources(wadg_ctx* ctx) {
   // no source counts until the new tables are complete
   ctx->nsrc = 0;
   ctx->src_ok = false;
-  std::vector<SrcDev> sd;
-  std::vector<Real> w, ws;
+  struct Place { int64_t k; double rst[3]; };
+  std::vector<Place> at;
+  std::vector<size_t> order;
   for (const wadg_dipole& d : ctx->src_user) {
-    double rst[3];
-    int64_t k = locate(ctx, d.x, rst);
-    if (k < 0)
+    Place p;
+    p.k = locate(ctx, d.x, p.rst);
+    if (p.k < 0)
       return fail(ctx, WADG_ENOTFOUND, "source point (%g, %g, %g) is outside the mesh", d.x[0],
                   d.x[1], d.x[2]);
+    order.push_back(at.size());
+    at.push_back(p);
+  }
+  // by (batch, element): a tile's sources are then one range of the table
+  std::stable_sort(order.begin(), order.end(), [&](size_t a, size_t b) {
+    const int ba = ctx->src_user[a].batch, bb = ctx->src_user[b].batch;
+    return ba != bb ? ba < bb : ctx->iperm[at[a].k] < ctx->iperm[at[b].k];
+  });
+  std::vector<SrcDev> sd;
+  std::vector<Real> w, ws;
+  for (size_t i : order) {
+    const wadg_dipole& d = ctx->src_user[i];
+    const int64_t k = at[i].k;
+    const double* rst = at[i].rst;
     std::vector<double> ell = ctx->ref.lagrange_at(rst[0], rst[1], rst[2]);
     SrcDev s{};
     s.elem = (int)ctx->iperm[k];

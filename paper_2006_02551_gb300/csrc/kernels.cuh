@@ -60,6 +60,8 @@ __host__ __device__ constexpr int quad_capacity(int N, int qc) {
   return qc ? compact_nq(N) : (N + 1) * (N + 1) * (N + 1);
 }
 
+// the sources' table is sorted by (batch, element): those of a tile follow one
+// another, and those of an element keep the caller's order
 struct SrcDev {
   int elem;     // internal element id
   int batch;

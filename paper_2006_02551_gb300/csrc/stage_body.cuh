@@ -63,7 +63,7 @@ struct Tile {
   static constexpr int t1 = t0 < t_tasks ? t0 : t_tasks;
   static constexpr int T = t1 < 1 ? 1 : (t1 > 32 ? 32 : t1);
   static constexpr size_t smem =
-      (size_t)(ops_sz + T * per_elem) * sizeof(Real) + 64 * sizeof(int);
+      (size_t)(ops_sz + T * per_elem) * sizeof(Real);
 };
 
 __device__ __forceinline__ double dipole_current(const SrcDev& s, double t) {
@@ -141,8 +141,7 @@ __device__ __forceinline__ void stage_body(const StageParams<Real>& P, unsigned 
   Real* RS = U + TE * TL::u_sz;      // [TE][NpP][6]
   Real* nrm = RS + TE * TL::r_sz;    // [TE][4][4]
   Real* met = nrm + TE * 16;         // [TE][12] (9 used)
-  int* srcl = reinterpret_cast<int*>(met + TE * 12);
-  __shared__ int nsl;
+  __shared__ int nsl, src0;          // the tile's sources: count, first of the table
 
   const unsigned char* Fmask = P.tabs;
   const unsigned char* fperm = P.tabs + NF;
@@ -177,7 +176,10 @@ __device__ __forceinline__ void stage_body(const StageParams<Real>& P, unsigned 
   __syncthreads();   // previous tile done with the shared buffers
 
   // ---- phase 0: fields (component-fastest), geometry, sources of the tile
-  if (tid == 0) nsl = 0;
+  if (tid == 0) {
+    nsl = 0;
+    src0 = P.nsrc;
+  }
   for (int idx = tid; idx < ne * 6 * Np; idx += NT) {
     const int e = idx / (6 * Np), r = idx - e * 6 * Np, c = r / Np, j = r - c * Np;
     F[(e * Np + j) * CF + c] = qin[(int64_t)eg0 * 6 * Np + idx];
@@ -197,8 +199,8 @@ __device__ __forceinline__ void stage_body(const StageParams<Real>& P, unsigned 
   for (int s = tid; s < P.nsrc; s += NT) {
     const SrcDev& sd = P.src[s];
     if (sd.batch == b && sd.elem >= eg0 && sd.elem < eg0 + ne) {
-      const int slot = atomicAdd(&nsl, 1);
-      if (slot < 64) srcl[slot] = s;
+      atomicAdd(&nsl, 1);
+      atomicMin(&src0, s);
     }
   }
 
@@ -250,7 +252,7 @@ __device__ __forceinline__ void stage_body(const StageParams<Real>& P, unsigned 
     fo[5] = sE * (YP * cEz + al * (nz * ndH - dHz));
   }
   __syncthreads();
-  const int nsrc_l = min(nsl, 64);
+  const int sb0 = src0, sb1 = sb0 + nsl;
 
   // ---- phases 2 and 3
   //   curl task (e, fld, iq): fld 0: Cbar(E) -> rhs_H = -Cbar(E)/mu,
@@ -324,14 +326,14 @@ __device__ __forceinline__ void stage_body(const StageParams<Real>& P, unsigned 
       else { out[0][n] = c0; out[1][n] = c1; out[2][n] = c2; }
     }
     if (fld == 1) {
-      for (int s = 0; s < nsrc_l; ++s) {
-        const SrcDev& sd = P.src[srcl[s]];
+      for (int s = sb0; s < sb1; ++s) {
+        const SrcDev& sd = P.src[s];
         if (sd.elem != eg) continue;
         const Real jt = (Real)dipole_current(sd, tst);
 #pragma unroll
         for (int n = 0; n < 4; ++n) {
           const int i = 4 * iq + n;
-          const Real w = i < Np ? P.src_w[srcl[s] * Np + i] : Real(0);
+          const Real w = i < Np ? P.src_w[(int64_t)s * Np + i] : Real(0);
 #pragma unroll
           for (int c = 0; c < 3; ++c) out[c][n] -= jt * (Real)sd.dir[c] * w;
         }

@@ -40,7 +40,7 @@ struct SaTile {
            al(te * 2 * UST) + al(te * 6 * NF) + te * NG * 12 + te * NG * 48 + al(te);
   }
   WADG_HD static constexpr size_t bytes(int te) {
-    return (size_t)floats(te) * 4 + te * 16 + 256 + tabB + 64;
+    return (size_t)floats(te) * 4 + te * 16 + tabB + 64;
   }
   static constexpr int fit() {   // two blocks per SM; one where four elements need it
     for (int t = 16; t > 4; --t)
@@ -284,15 +284,14 @@ sym_adj_kernel(const AdjParams<float> A,
   float* ZV = SG + TE * ST::NG * 12;                        // [ng][8][6 TE] point values
   float* GE = ZV + TE * ST::NG * 48;                        // [TE] dJ/deps_k
   int* nbr = reinterpret_cast<int*>(smem_raw + (size_t)ST::floats(TE) * 4);
-  int* srcl = nbr + TE * 4;
-  unsigned char* tab = reinterpret_cast<unsigned char*>(srcl + 64);
+  unsigned char* tab = reinterpret_cast<unsigned char*>(nbr + TE * 4);
   uint64_t* bar = reinterpret_cast<uint64_t*>(tab + ST::tabB);
   const unsigned char* t_or = tab + 8 * Nfp;
   const unsigned char* t_nf = tab + 8 * Nfp + 4 * B::NFul + 8;   // [Np][3] face nodes, NF: none
   const unsigned char* Fmask = tab + ST::TAB;
   const unsigned char* fperm = Fmask + NF;
   const unsigned char* fmap = fperm + 96 * Nfp;
-  __shared__ int nsl;
+  __shared__ int nsl, src0;   // the tile's sources: count, first of the table
   __shared__ double red[6][NT / 32];
   const int tid = threadIdx.x;
   const uint32_t mb = tc::saddr(bar);
@@ -311,6 +310,7 @@ sym_adj_kernel(const AdjParams<float> A,
     tc::mbar_init(mb, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     nsl = 0;
+    src0 = A.nsrc;
     const void* src[6] = {A.nbr + (int64_t)eg0 * 4, A.facex + (int64_t)eg0 * 32, A.q_in + oq,
                           A.geox + (int64_t)eg0 * 12, nullptr, nullptr};
     uint32_t len[6] = {(uint32_t)ne * 16, (uint32_t)ne * 128, (uint32_t)(ne * 6 * Np * 4),
@@ -362,8 +362,8 @@ sym_adj_kernel(const AdjParams<float> A,
   for (int s = tid; s < A.nsrc; s += NT) {
     const SrcDev& sd = A.src[s];
     if (sd.batch == b && sd.elem >= eg0 && sd.elem < eg0 + ne) {
-      const int slot = atomicAdd(&nsl, 1);
-      if (slot < 64) srcl[slot] = s;
+      atomicAdd(&nsl, 1);
+      atomicMin(&src0, s);
     }
   }
   // ---- traces: the transposed upwind flux of both sides of each face node,
@@ -453,7 +453,7 @@ sym_adj_kernel(const AdjParams<float> A,
   // ---- adapted sums of mu (scaled by 1/eps, -1/mu below: element constants)
   adapt_rows<N, UST>(MQ, t_or, U, ne, tid, NT);
   __syncthreads();
-  const int nsrc_l = min(nsl, 64);
+  const int sb0 = src0, sb1 = sb0 + nsl;
   // ---- curl^T: warps 0-3 take the four characters; E rows act on H and H
   // rows on E (TE <= 16: one lane per element and field)
   {
@@ -607,13 +607,13 @@ sym_adj_kernel(const AdjParams<float> A,
     }
   }
   // source term of dJ/deps_k: + mu_E . J / eps^2
-  for (int k = 0; k < nsrc_l; ++k) {
-    const SrcDev& sd = A.src[srcl[k]];
+  for (int s = sb0; s < sb1; ++s) {
+    const SrcDev& sd = A.src[s];
     const int e = sd.elem - eg0;
     const float ie = GX[e * 12 + 10];
     const float jt = (float)dipole_current(sd, A.t) * ie * ie;
     for (int i = tid; i < 3 * Np; i += NT)
-      atomicAdd(&GE[e], jt * (float)sd.dir[i / Np] * A.src_w[srcl[k] * Np + i % Np] *
+      atomicAdd(&GE[e], jt * (float)sd.dir[i / Np] * A.src_w[(int64_t)s * Np + i % Np] *
                             MQ[e * 6 * Np + i]);
   }
   // ---- lambda_in = lambda_out + dt L^T mu, rho_prev = A_i mu (all loads first)

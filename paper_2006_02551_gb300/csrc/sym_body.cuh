@@ -134,9 +134,9 @@ struct SymTile {
     return ops + fieldsR(te) + te * 12 + te * 64 + al(te * 2 * UST) + fluxR(te) + sigR(te) +
            (s - 1) * te * 12 * Np;
   }
-  // + neighbours, source list, tables, barriers
+  // + neighbours, tables, barriers
   WADG_HD static constexpr size_t bytes(int te, int s) {
-    return (size_t)reals(te, s) * RS + te * 32 + 256 + tabB + 64;
+    return (size_t)reals(te, s) * RS + te * 32 + tabB + 64;
   }
   static constexpr size_t kMax = 226 * 1024;
   static constexpr int blocks(int te) {   // that fit an SM, of the two wanted
@@ -665,14 +665,13 @@ __device__ __forceinline__ void sym_body(const StageParams<Real>& P, const SymCo
   Real* SG = FL + ST::fluxR(TE);                  // sigma [TE][ng][3][4], then kappa
   Real* PS = SG + ST::sigR(TE);                   // [S - 1][TE * 12][Np] partial sums
   int* nbr2 = reinterpret_cast<int*>(ops + ST::reals(TE, S));   // 2 x [TE][4]
-  int* srcl = nbr2 + TE * 8;                      // [64]
-  unsigned char* tab = reinterpret_cast<unsigned char*>(srcl + 64);
+  unsigned char* tab = reinterpret_cast<unsigned char*>(nbr2 + TE * 8);
   uint64_t* bar = reinterpret_cast<uint64_t*>(tab + ST::tabB);
   const unsigned char* t_fm = tab;                // [Nfp][4] face node
   const unsigned char* t_fn = tab + 4 * Nfp;      // [Nfp][4] volume node
   const unsigned char* t_or = tab + 8 * Nfp;      // node orbits
   const unsigned char* fperm = tab + ST::TAB + NF;
-  __shared__ int nsl, dyn_tile;
+  __shared__ int nsl, src0, dyn_tile;   // the tile's sources: count, first of the table
   const int tid = threadIdx.x;
 
   for (int i = tid; i < ST::ops / 2; i += NT) {
@@ -756,6 +755,7 @@ __device__ __forceinline__ void sym_body(const StageParams<Real>& P, const SymCo
     const int fb = phase & 1;
     if (tid == 0) {
       nsl = 0;
+      src0 = P.nsrc;
       const void* src[5] = {P.qin + oq, P.geox + (int64_t)eg0 * 12, nullptr, nullptr, nullptr};
       uint32_t len[5] = {(uint32_t)(ne * 6 * Np * sizeof(Real)),
                          (uint32_t)(ne * 12 * sizeof(Real)), 0, 0, 0};
@@ -839,8 +839,8 @@ __device__ __forceinline__ void sym_body(const StageParams<Real>& P, const SymCo
     for (int s = tid; s < P.nsrc; s += NT) {
       const SrcDev& sd = P.src[s];
       if (sd.batch == b && sd.elem >= eg0 && sd.elem < eg0 + ne) {
-        const int slot = atomicAdd(&nsl, 1);
-        if (slot < 64) srcl[slot] = s;
+        atomicAdd(&nsl, 1);
+        atomicMin(&src0, s);
       }
     }
 
@@ -998,19 +998,19 @@ __device__ __forceinline__ void sym_body(const StageParams<Real>& P, const SymCo
         sym_curl_pairs<N, 1, ST::CC>(ops, x, uu, ff, g, sc, out);
       }
     }
-    const int nsrc_l = min(nsl, 64);
+    const int sb0 = src0, sb1 = sb0 + nsl;
     __syncthreads();
-    if (nsrc_l) {   // dipole sources: adapted coefficients of M_k^-1 l(r_s)
-      for (int k = 0; k < nsrc_l; ++k) {
-        const SrcDev& sd = P.src[srcl[k]];
+    if (sb1 > sb0) {   // dipole sources: adapted coefficients of M_k^-1 l(r_s)
+      for (int s = sb0; s < sb1; ++s) {   // (a thread keeps its values of an element)
+        const SrcDev& sd = P.src[s];
         const int e = sd.elem - eg0;
         const Real jt = (Real)dipole_current(sd, tst) * GX[e * 12 + 10];
         for (int i = tid; i < 3 * Np; i += NT) {
           const int c = i / Np;
-          U[e * 2 * UST + i] -= jt * (Real)sd.dir[c] * P.src_ws[srcl[k] * Np + i - c * Np];
+          U[e * 2 * UST + i] -= jt * (Real)sd.dir[c] * P.src_ws[(int64_t)s * Np + i - c * Np];
         }
-        __syncthreads();
       }
+      __syncthreads();
     }
 
     if constexpr (!PML) {

@@ -107,9 +107,9 @@ struct Plan {
   // the current tile's metric (9) and 1/eps, 1/mu in float [T][12]
   static constexpr uint32_t oST = oGeo + ((T * 12 * 4 + 15) & ~15u);  // two staging sets
   static constexpr uint32_t oMisc = oST + 2 * SET;
-  // misc: 10 mbarriers | TMEM slot | flags | tile source list (64) | cached
+  // misc: 10 mbarriers | TMEM slot | the tile's sources (2) | cached
   // (batch, element) of the first 64 sources | face tables (Fmask, fperm)
-  static constexpr uint32_t oTabs = 896;
+  static constexpr uint32_t oTabs = 640;
   static constexpr uint32_t MISC_BYTES = (oTabs + 100 * Nfp + 15) & ~15u;
   // epilogue scratch: the node rows of the products copied out of TMEM so that
   // every warp can share the per-node work.  PML: the volume/LIFT columns go
@@ -211,9 +211,8 @@ __global__ void __launch_bounds__(TcWarps<N, BF>::threads,
   // [7], [8] staging set 0 / 1 landed
   uint64_t* mbar = reinterpret_cast<uint64_t*>(smem + PL::oMisc);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + PL::oMisc + 80);
-  int* flags = reinterpret_cast<int*>(smem + PL::oMisc + 84);   // [0] source count
-  int* srcl = reinterpret_cast<int*>(smem + PL::oMisc + 112);
-  int* srcc = reinterpret_cast<int*>(smem + PL::oMisc + 368);   // [64][2] batch, element
+  int* srct = reinterpret_cast<int*>(smem + PL::oMisc + 84);    // the tile's sources: count, first
+  int* srcc = reinterpret_cast<int*>(smem + PL::oMisc + 112);   // [64][2] batch, element
   constexpr int kSrcCache = 64;
   const float* tops = reinterpret_cast<const float*>(P.tcops);
   // face-node tables, copied to shared memory in the prologue: Fmask [NF],
@@ -543,7 +542,10 @@ __global__ void __launch_bounds__(TcWarps<N, BF>::threads,
     float* pio = P.p + (int64_t)b * P.strideP;
     float* resp = P.resp + (int64_t)b * P.strideP;
 
-    if (tid == 0) flags[0] = 0;
+    if (tid == 0) {
+      srct[0] = 0;
+      srct[1] = P.nsrc;
+    }
     if (next < ntiles) {
       load_nbr_idx(next, nbv, codev);   // consumed after this tile's flux
     }
@@ -563,8 +565,8 @@ __global__ void __launch_bounds__(TcWarps<N, BF>::threads,
       const int sb = s < kSrcCache ? srcc[2 * s] : P.src[s].batch;
       const int se = s < kSrcCache ? srcc[2 * s + 1] : P.src[s].elem;
       if (sb == b && se >= eg0 && se < eg0 + ne) {
-        const int slot = atomicAdd(&flags[0], 1);
-        if (slot < 64) srcl[slot] = s;
+        atomicAdd(&srct[0], 1);
+        atomicMin(&srct[1], s);
       }
     }
     // ---- B operand of the field products (TF32-rounded), from the staged
@@ -720,7 +722,7 @@ __global__ void __launch_bounds__(TcWarps<N, BF>::threads,
     if (next < ntiles) load_sig(next, sgv);
     signal_ready(5);   // P_q operand; the product overlaps the epilogue below
     if (!wait_bar(1)) { failed = true; break; }
-    const int nsrc_l = min(flags[0], 64);
+    const int sb0 = srct[1], sb1 = sb0 + srct[0];
 
     // ---- derivative and LIFT columns -> shared memory.  Lane d Np + i holds
     // the d-th derivative at node i, lane i the LIFT term at node i.
@@ -809,13 +811,13 @@ __global__ void __launch_bounds__(TcWarps<N, BF>::threads,
       CE[0] = dy[2] - dz[1] + lf[3];
       CE[1] = dz[0] - dx[2] + lf[4];
       CE[2] = dx[1] - dy[0] + lf[5];
-      for (int s = 0; s < nsrc_l; ++s) {
-        const SrcDev& sd = P.src[srcl[s]];
+      for (int s = sb0; s < sb1; ++s) {
+        const SrcDev& sd = P.src[s];
         if (sd.elem != eg) continue;
         const double tau = sd.width;
         const double gg = exp(-(tst - sd.t0) * (tst - sd.t0) / (4.0 * tau * tau));
         const float jt = (float)(sd.amp * (-(tst - sd.t0) / (2.0 * tau * tau)) * gg);
-        const float w = P.src_w[srcl[s] * Np + i];
+        const float w = P.src_w[(int64_t)s * Np + i];
 #pragma unroll
         for (int c = 0; c < 3; ++c) CH[c] -= jt * (float)sd.dir[c] * w;
       }

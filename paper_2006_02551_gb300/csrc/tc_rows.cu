@@ -807,7 +807,7 @@ __global__ void __launch_bounds__(RPlan<N, PML, BF>::THREADS, 1)
 #pragma unroll
           for (int ic = 0; ic < NHC; ++ic)
             if (i0 + ic < i1)
-              rhs[ic] -= PML ? ie * jt * P.src_w[s * Np + i0 + ic] : jt * P.src_w[s * Np + i0 + ic];
+              rhs[ic] -= PML ? ie * jt * P.src_w[(int64_t)s * Np + i0 + ic] : jt * P.src_w[(int64_t)s * Np + i0 + ic];
         }
       }
       // the non-PML class scales the curl and the source together, as the
