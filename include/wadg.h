@@ -449,7 +449,10 @@ wadg_status wadg_group_info(const wadg_group* g, int32_t* nblocks, int32_t* thre
  * wadg_run_steps.  Gives each member the values wadg_run_steps would.  The
  * members are packed into clusters whose per-step device data fits half of
  * the L2 (members above that form one cluster); each cluster runs all nsteps
- * before the next, so small members step out of L2. */
+ * before the next, so small members step out of L2.  WADG_ETIMEOUT where a
+ * bounded device-side wait of a member's launch gave up (the message names the
+ * member; its state is partly updated, and members of later clusters have not
+ * stepped). */
 wadg_status wadg_group_run_steps(wadg_group* g, int64_t nsteps, const double* dt,
                                  double* const* probe_out);
 

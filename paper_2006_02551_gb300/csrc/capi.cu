@@ -975,7 +975,17 @@ wadg_status capture_graphs(wadg_ctx* ctx, double dt) {
   return WADG_OK;
 }
 
-// bounded device waits that gave up leave a flag behind
+// bounded device waits that gave up leave a flag behind: the status of flag
+// word e of a context
+wadg_status flag_status(int e, const char** text) {
+  if (e & 1) {
+    *text = "a stage kernel gave up waiting for its copies or products";
+    return WADG_ETIMEOUT;
+  }
+  *text = "a device index check failed (checked build): mesh tables corrupt";
+  return WADG_ECUDA;
+}
+
 wadg_status check_err_flag(wadg_ctx* ctx) {
   int e = 0;
   CK(cudaMemcpyAsync(&e, ctx->errflag.p, 4, cudaMemcpyDeviceToHost, ctx->stream));
@@ -983,9 +993,9 @@ wadg_status check_err_flag(wadg_ctx* ctx) {
   CK(cudaStreamSynchronize(ctx->stream));
   if (e) {
     CK(cudaMemset(ctx->errflag.p, 0, 4));
-    if (e & 1)
-      return fail(ctx, WADG_ETIMEOUT, "a tensor-core stage kernel gave up waiting for its products");
-    return fail(ctx, WADG_ECUDA, "a device index check failed (checked build): mesh tables corrupt");
+    const char* text = nullptr;
+    const wadg_status s = flag_status(e, &text);
+    return fail(ctx, s, "%s", text);
   }
   return WADG_OK;
 }
@@ -2224,6 +2234,8 @@ struct wadg_group {
   // hold every member.
   std::vector<std::vector<int>> cluster_of;
   std::vector<wadg_group*> clusters;
+  std::vector<int> ids;   // a cluster: its members' places in the user's group
+  int* flags = nullptr;   // pinned: the members' error flags after a call
 };
 
 namespace {
@@ -2245,6 +2257,31 @@ wadg_status gfail(wadg_group* g, wadg_status s, const char* fmt, ...) {
       return gfail(g, e_ == cudaErrorMemoryAllocation ? WADG_ENOMEM : WADG_ECUDA,       \
                    "%s: %s", #call, cudaGetErrorString(e_));                            \
   } while (0)
+
+// The members' error flags: the copies to the host, issued behind the launches
+// they report on, and, with the stream idle, the status of the first one set
+// (all are cleared).
+cudaError_t group_read_flags(wadg_group* g) {
+  for (size_t c = 0; c < g->ctx.size(); ++c) {
+    const cudaError_t e = cudaMemcpyAsync(g->flags + c, g->ctx[c]->errflag.p, 4,
+                                          cudaMemcpyDeviceToHost, g->stream);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+wadg_status group_check_flags(wadg_group* g) {
+  wadg_status s = WADG_OK;
+  for (size_t c = 0; c < g->ctx.size(); ++c) {
+    if (!g->flags[c]) continue;
+    GCK(cudaMemsetAsync(g->ctx[c]->errflag.p, 0, 4, g->stream));
+    if (s != WADG_OK) continue;
+    const char* text = nullptr;
+    s = flag_status(g->flags[c], &text);
+    gfail(g, s, "member %d: %s", g->ids.empty() ? (int)c : g->ids[c], text);
+  }
+  if (s != WADG_OK) GCK(cudaStreamSynchronize(g->stream));
+  return s;
+}
 
 // every member's device tables are complete (no set-up call of a member
 // failed part-way since its last success)
@@ -2589,6 +2626,7 @@ wadg_status wadg_group_create(int32_t n, wadg_ctx* const* ctxs, wadg_group** out
   cudaDeviceGetAttribute(&g->sms, cudaDevAttrMultiProcessorCount, g->device);
   if (g->sms < 1) g->sms = 1;
   cudaError_t e = configure_group_kernel();
+  if (e == cudaSuccess) e = cudaMallocHost(&g->flags, (size_t)n * sizeof(int));
   if (e != cudaSuccess) {
     delete g;
     return fail(nullptr, WADG_ECUDA, "group kernel set-up: %s", cudaGetErrorString(e));
@@ -2610,6 +2648,7 @@ wadg_status wadg_group_destroy(wadg_group* g) {
   dfree(g->dcounter);
   for (cudaStream_t st : g->aux) cudaStreamDestroy(st);
   for (cudaEvent_t e : g->ev) cudaEventDestroy(e);
+  cudaFreeHost(g->flags);
   delete g;
   return WADG_OK;
 }
@@ -2668,7 +2707,9 @@ wadg_status wadg_group_autotune(wadg_group* g, const double* dt, int32_t reps, d
   g->per_item = best_item;
   group_plan(g);
   if (ms_out) *ms_out = best / reps;
-  return WADG_OK;
+  GCK(group_read_flags(g));
+  GCK(cudaStreamSynchronize(g->stream));
+  return group_check_flags(g);
 }
 
 wadg_status wadg_group_set_tuning(wadg_group* g, int32_t per_item, int32_t parallel,
@@ -2733,6 +2774,7 @@ wadg_status wadg_group_run_steps(wadg_group* g, int64_t nsteps, const double* dt
         return gfail(g, s0, "cluster set-up: %s", wadg_group_last_error(nullptr));
       }
       sub->stream = g->stream;
+      sub->ids = c;
       g->clusters.push_back(sub);
     }
     g->cluster_of = cl;
@@ -2810,6 +2852,7 @@ wadg_status wadg_group_run_steps(wadg_group* g, int64_t nsteps, const double* dt
         GCK(cudaMemcpyAsync(probe_out[c] + (size_t)done * rec, x->pr_out.p, (size_t)n * rec * 8,
                             cudaMemcpyDeviceToHost, g->stream));
     }
+    if (done + n == nsteps) GCK(group_read_flags(g));
     GCK(cudaStreamSynchronize(g->stream));
     done += n;
   }
@@ -2818,7 +2861,7 @@ wadg_status wadg_group_run_steps(wadg_group* g, int64_t nsteps, const double* dt
     x->t += nsteps * dt[c];
     if (nsteps & 1) x->cur ^= 1;   // each step flips the buffers once
   }
-  return WADG_OK;
+  return group_check_flags(g);
 }
 
 const char* wadg_group_last_error(const wadg_group* g) {
