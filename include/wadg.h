@@ -341,20 +341,23 @@ wadg_status wadg_synchronize(wadg_ctx* ctx);
  * (wadg_group_*) do not count.  (The paper has no counterpart.) */
 wadg_status wadg_set_memory_limit(wadg_ctx* ctx, size_t bytes, size_t* held_out);
 
-/* Failure-detection test aid for the TF32 and BF16 contexts, the ones whose
- * kernels wait on device-side signals (the mbarriers between the tensor-core
- * issuing thread and the compute warps).  Every such wait gives up after
- * about one second, sets the context's error flag and lets the kernel drain
- * the products it issued, release its tensor memory and end; the call that
- * launched it (wadg_rk_stage, wadg_run_steps, wadg_run_steps_noalloc) then
- * returns WADG_ETIMEOUT, with the state partly updated.  This call arms one
+/* Failure-detection test aid.  The stage kernels wait on device-side signals:
+ * the mbarriers of their bulk copies and, in TF32 and BF16 contexts, those
+ * between the tensor-core issuing thread and the compute warps.  Every such
+ * wait gives up after about one second, sets the context's error flag and lets
+ * the kernel drain what it issued, release its tensor memory and end; the call
+ * that launched it (wadg_rk_stage, wadg_run_steps, wadg_run_steps_noalloc,
+ * wadg_adjoint, wadg_group_run_steps) then returns WADG_ETIMEOUT, with the state
+ * partly updated.  This call arms one
  * request: the first block of a later tensor-core stage launch that takes it
  * issues the flux product of its first tile without the completion signal,
  * so that one wait runs out.  Nothing faults, traps or waits without limit,
  * and the context stays usable (set the state again and step).  The request
  * stays armed until a launch takes it.  EUNSUPPORTED for FP64 and FP32
- * contexts.  (The paper has no counterpart; this tests the library's error
- * path.) */
+ * contexts, except in the diagnostic build (-DWADG_CHECKED), whose FP64 and FP32
+ * kernels take the request by waiting for bytes that no copy brings; two calls
+ * in a row arm the FP32 reverse stage of wadg_adjoint there.  (The paper has no
+ * counterpart; this tests the library's error path.) */
 wadg_status wadg_arm_wait_timeout(wadg_ctx* ctx);
 
 /* Measured fused multiply-add throughput of device `device`'s CUDA cores in

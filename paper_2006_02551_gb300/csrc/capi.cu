@@ -147,6 +147,14 @@ struct wadg_ctx {
 
 namespace {
 
+// whether this is the diagnostic build (device-side index checks, time-outs that
+// can be armed on the CUDA-core kernels)
+#ifdef WADG_CHECKED
+constexpr bool kDiagnostic = true;
+#else
+constexpr bool kDiagnostic = false;
+#endif
+
 wadg_status fail(wadg_ctx* c, wadg_status s, const char* fmt, ...) {
   char buf[512];
   va_list ap;
@@ -801,7 +809,7 @@ StageParams<Real> stage_params(wadg_ctx* ctx, int stage, double dt, double t, bo
   }
   P.tcops = ctx->tcops.p;
   P.err = (int*)ctx->errflag.p;
-  P.inject = ctx->tc ? (int*)ctx->errflag.p + 1 : nullptr;
+  P.inject = ctx->tc || kDiagnostic ? (int*)ctx->errflag.p + 1 : nullptr;
   return P;
 }
 
@@ -1844,6 +1852,7 @@ wadg_status adjoint_typed(wadg_ctx* ctx, int64_t nsteps, double dt, int C, doubl
   A.symadj = (const Real*)ctx->symadj.p; A.symtab = (const unsigned char*)ctx->symtab.p;
   A.geox = (const Real*)ctx->geox.p; A.facex = (const Real*)ctx->facex.p;
   A.err = (int*)ctx->errflag.p;
+  A.inject = kDiagnostic ? (int*)ctx->errflag.p + 1 : nullptr;
   for (int u = 0; u < 3; ++u) {
     A.sigma_max[u] = ctx->has_prof ? ctx->prof.sigma_max[u] : 0.0;
     A.p_sigma[u] = ctx->has_prof ? ctx->prof.p_sigma[u] : 0.0;
@@ -2004,11 +2013,19 @@ wadg_status wadg_set_memory_limit(wadg_ctx* ctx, size_t bytes, size_t* held_out)
 
 wadg_status wadg_arm_wait_timeout(wadg_ctx* ctx) {
   if (!ctx) return fail(nullptr, WADG_EINVAL, "null context");
-  if (!ctx->tc)
-    return fail(ctx, WADG_EUNSUPPORTED, "only the tensor-core kernels wait on device-side signals");
+  if (!ctx->tc && !kDiagnostic)
+    return fail(ctx, WADG_EUNSUPPORTED,
+                "a time-out is armed on TF32 and BF16 contexts (on FP64 and FP32 ones in the "
+                "diagnostic build only)");
   cudaSetDevice(ctx->device);
-  const int one = 1;
-  CK(cudaMemcpyAsync((int*)ctx->errflag.p + 1, &one, 4, cudaMemcpyHostToDevice, ctx->stream));
+  int kind = kRequestStage;
+  if (!ctx->tc) {   // a second call in a row: the reverse stage
+    int held = 0;
+    CK(cudaMemcpyAsync(&held, (int*)ctx->errflag.p + 1, 4, cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaStreamSynchronize(ctx->stream));
+    if (held) kind = kRequestReverse;
+  }
+  CK(cudaMemcpyAsync((int*)ctx->errflag.p + 1, &kind, 4, cudaMemcpyHostToDevice, ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
   return WADG_OK;
 }

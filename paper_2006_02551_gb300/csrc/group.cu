@@ -44,7 +44,7 @@ group_stage_kernel(const GroupParams G,
     }
     __syncthreads();
     if (!go) continue;
-    sym_body<float, N, PML ? 2 : 0, KAPPA>(P, C, smem_raw, 0, 1, G.counter + it);
+    if (!sym_body<float, N, PML ? 2 : 0, KAPPA>(P, C, smem_raw, 0, 1, G.counter + it)) return;
   }
 }
 

@@ -48,6 +48,20 @@ __device__ __forceinline__ bool wadg_index_ok(bool ok, int* status) {
 #define WADG_INDEX_OK(cond, status) true
 #endif
 
+// Diagnostic build: whether this thread takes a failure-detection request armed
+// for its kind of kernel (kRequestStage, kRequestReverse).  The block that does
+// tells its copy barrier of bytes that no copy brings, so that its bounded wait
+// runs out.
+constexpr int kRequestStage = 1, kRequestReverse = 2;
+#ifdef WADG_CHECKED
+__device__ __forceinline__ bool wadg_take_request(int* request, int kind) {
+  return request && *reinterpret_cast<volatile int*>(request) == kind &&
+         atomicCAS(request, kind, 0) == kind;
+}
+#else
+__device__ __forceinline__ bool wadg_take_request(int*, int) { return false; }
+#endif
+
 // Volume quadrature capacity of the PML stage kernels (eqs. 20, 21, 26-29).
 // Class 0: the default conical-product rule of (N+1)^3 points.  Class 1:
 // compact rules of degree 2N of at most compact_nq(N) points (a rule with
@@ -113,7 +127,7 @@ struct StageParams {
   int split;                // threads that share a row's groups (sym_split)
   const void* tcops;        // tensor-core operator tables (TF32 path)
   int* err;                 // device error flag (bounded waits that gave up)
-  int* inject;              // tensor-core kernels: armed failure-detection request
+  int* inject;              // armed failure-detection request (FP64, FP32: diagnostic build)
                             // (nonzero: one block withholds a product signal), or null
 };
 
@@ -135,6 +149,7 @@ struct AdjParams {
   const Real* geox;
   const Real* facex;
   int* err;                 // device error flag (bounded waits that gave up)
+  int* inject;              // armed failure-detection request (diagnostic build)
   int tile;                 // elements per tile (set by the launcher)
   const double* geo;
   const Real* fnrm;         // [e][4][4]: unit outward normal, Fscale (as the forward stage)

@@ -322,7 +322,7 @@ sym_adj_kernel(const AdjParams<float> A,
       src[n] = A.sig + (int64_t)ep0 * ng * 12; len[n] = (uint32_t)ne * ng * 48;
       dst[n++] = tc::saddr(SG);
     }
-    uint32_t total = 0;
+    uint32_t total = wadg_take_request(A.inject, kRequestReverse) ? 16 : 0;
     for (int a = 0; a < n; ++a) {
       const uint32_t lo = (uint32_t)(reinterpret_cast<uintptr_t>(src[a]) & 15);
       len[a] = (lo + len[a] + 15) & ~15u;

@@ -638,9 +638,10 @@ __device__ __forceinline__ void sym_to_sums(Real* s) {
 
 // One element class of one context; smem_raw is the block's dynamic shared
 // memory.  Tiles by a static schedule, or from the counter *dyn (grouped
-// launch), as stage_body.
+// launch).  False where a copy did not land in time: the block then takes no
+// more tiles.
 template <typename Real, int N, int G, bool KAPPA, typename ST = SymTile<Real, N, G, KAPPA>>
-__device__ __forceinline__ void sym_body(const StageParams<Real>& P, const SymCoef<ST::coefs>& C,
+__device__ __forceinline__ bool sym_body(const StageParams<Real>& P, const SymCoef<ST::coefs>& C,
                                          unsigned char* smem_raw, int bid, int nblk,
                                          int* dyn = nullptr) {
   using B = Blocks<N, 4>;
@@ -705,9 +706,10 @@ __device__ __forceinline__ void sym_body(const StageParams<Real>& P, const SymCo
     return dyn_tile;
   };
   // copies of n global blocks (16-byte covers) completing on barrier m
+  // (withheld: bytes that the barrier waits for and no copy brings)
   auto copy_in = [&](const void* const* src, const uint32_t* len, const uint32_t* dst, int n,
-                     uint32_t m) {
-    uint32_t total = 0;
+                     uint32_t m, uint32_t withheld) {
+    uint32_t total = withheld;
     for (int a = 0; a < n; ++a)
       total += ((uint32_t)(reinterpret_cast<uintptr_t>(src[a]) & 15) + len[a] + 15) & ~15u;
     tc::fence_async_smem();   // earlier reads of the buffers come before the copies
@@ -725,7 +727,7 @@ __device__ __forceinline__ void sym_body(const StageParams<Real>& P, const SymCo
     const void* src[2] = {P.nbr + e0 * 4, P.facex + e0 * 32};
     const uint32_t len[2] = {(uint32_t)(n * 16), (uint32_t)(n * 32 * sizeof(Real))};
     const uint32_t dst[2] = {tc::saddr(nbr2 + fb * TE * 4), tc::saddr(FC2 + fb * TE * 32)};
-    copy_in(src, len, dst, 2, mf);
+    copy_in(src, len, dst, 2, mf, 0);
   };
   uint32_t phase = 0;   // tiles done: the barriers' parities
   bool failed = false, ahead = !dyn && bid < ntiles;   // ahead: this tile's faces are on their way
@@ -771,7 +773,7 @@ __device__ __forceinline__ void sym_body(const StageParams<Real>& P, const SymCo
         }
       }
       if (!ahead) faces_in(tile, fb);
-      copy_in(src, len, dst, n, mb);
+      copy_in(src, len, dst, n, mb, wadg_take_request(P.inject, kRequestStage) ? 16 : 0);
       // the registers the update reads, and the next tile, into L2 meanwhile
       auto pre = [&](const Real* p, int n_) {
         const uintptr_t a = reinterpret_cast<uintptr_t>(p) & ~uintptr_t(15);
@@ -1382,6 +1384,7 @@ __device__ __forceinline__ void sym_body(const StageParams<Real>& P, const SymCo
     asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(mf) : "memory");
   }
   __syncthreads();
+  return !failed;
 }
 
 }  // namespace wadg

@@ -359,9 +359,10 @@ class Solver:
         return held.value
 
     def arm_wait_timeout(self):
-        """Failure-detection test aid (TF32/BF16 contexts): the next
-        tensor-core stage launch withholds one product signal, its bounded
-        wait runs out and the stepping call raises WadgError(ETIMEOUT)."""
+        """Failure-detection test aid (TF32/BF16 contexts; any context of the
+        diagnostic build): the next stage launch withholds one signal, its
+        bounded wait runs out and the stepping call raises
+        WadgError(ETIMEOUT)."""
         self._c(self.lib.wadg_arm_wait_timeout(self.ctx))
 
 
