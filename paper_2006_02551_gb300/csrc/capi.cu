@@ -282,6 +282,7 @@ wadg_status upload_sym(wadg_ctx* ctx) {
   std::vector<unsigned char> tab;
   build_sym_tables(R, ctx->sym, ops, tab);
   const int G = ctx->sym.G;
+  const size_t pq_end = ops.size();
   ctx->symcoef.clear();
   if (G)
     ctx->symcoef.assign(ops.end() - 2 * sample_groups(ctx) * sym_cp(R.N, G), ops.end());
@@ -292,7 +293,12 @@ wadg_status upload_sym(wadg_ctx* ctx) {
   CK(dalloc(ctx->symops, hr.size() * sizeof(Real)));
   CK(cudaMemcpy(ctx->symops.p, hr.data(), hr.size() * sizeof(Real), cudaMemcpyHostToDevice));
   if (sizeof(Real) == 4) {   // the adjoint's transposed blocks
-    const std::vector<float> tr = sym_transposed(R.N, ops);
+    std::vector<float> tr = sym_transposed(R.N, ops);
+    const size_t nc = ctx->symcoef.size();   // then what FP32 leaves of P_q
+    for (size_t k = nc / 2; k < nc; ++k) {
+      const double c = ops[pq_end - nc + k];
+      tr.push_back((float)(c - (double)(float)c));
+    }
     CK(dalloc(ctx->symadj, tr.size() * 4));
     CK(cudaMemcpy(ctx->symadj.p, tr.data(), tr.size() * 4, cudaMemcpyHostToDevice));
   }

@@ -144,7 +144,7 @@ struct AdjParams {
   double* grad_eps;         // [b][K] internal order
   double* grad_prof;        // [b][6]: d/dsigma_max[3], d/dp_sigma[3]
   // FP32, symmetric kernels (sym_adjoint.cu)
-  const Real* symadj;       // transposed derivative blocks, LIFT^T blocks
+  const Real* symadj;       // transposed derivative blocks, LIFT^T blocks, low parts of P_q
   const unsigned char* symtab;
   const Real* geox;
   const Real* facex;

@@ -31,6 +31,16 @@ struct SaTile {
   static constexpr int NG = PML ? sym_groups(N, G) : 0, CP = PML ? sym_cp(N, G) : 0;
   static constexpr int UST = 3 * Np | 1;
   static constexpr int DT = L::oL;            // transposed derivative blocks
+  // Low parts of P_q's coefficients (what FP32 rounds off), in the place of the
+  // derivative blocks once these are spent.  A V4 rule's P_q has a few hundred
+  // coefficients, whose roundings every element repeats, so that they add up over
+  // a mesh in the profile derivatives: median relative error of dJ/dsigma_max, N =
+  // 4, 16,464 tets, 8.3e-7 without the low parts, 3.8e-7 with them, 3.3e-7 in the
+  // dense kernel with its 48 times 35 coefficients (N = 5, 6,000 tets: 3.3e-6,
+  // 2.3e-6, 2.3e-6).  A gradient takes 1.2 % longer for them (N = 3, 82,944 tets).  Z2 rules have
+  // several times as many coefficients and the dense kernel's errors.
+  static constexpr int LO = G == 4 ? NG * CP : 0, LOT = (LO + kSaThreads - 1) / kSaThreads;
+  static_assert(LO <= DT, "low parts of P_q");
   static constexpr int TAB = 8 * Nfp + 4 * B::NFul + 8 + 3 * Np;
   static constexpr int tabB = (TAB + NF + 192 * Nfp + 15) & ~15;
   WADG_HD static constexpr int al(int x) { return (x + 3) & ~3; }
@@ -333,6 +343,12 @@ sym_adj_kernel(const AdjParams<float> A,
     for (int a = 0; a < n; ++a) tc::bulk_g2s(dst[a], src[a], len[a], mb);
   }
   for (int i = tid; i < ST::DT; i += NT) ops[i] = A.symadj[i];
+  float low[ST::LOT ? ST::LOT : 1];
+#pragma unroll
+  for (int k = 0; k < ST::LOT; ++k) {
+    const int i = tid + k * NT;
+    low[k] = i < ng * ST::CP ? A.symadj[L::oL + Np * ((Nfp + 3) & ~3) + i] : 0.f;
+  }
   for (int i = tid; i < ST::TAB; i += NT) tab[i] = A.symtab[i];
   for (int i = tid; i < NF + 192 * Nfp; i += NT) tab[ST::TAB + i] = A.tabs[i];
   for (int i = tid; i < TE; i += NT) GE[i] = 0.f;
@@ -470,6 +486,9 @@ sym_adj_kernel(const AdjParams<float> A,
     else if (y == 0) sym_curlt_pairs<N, 0>(ops, 0, U + r * UST, gs, out);
     else sym_curlt_pairs<N, 1>(ops, y, U + r * UST, gs, out);
   }
+#pragma unroll
+  for (int k = 0; k < ST::LOT; ++k)   // (the derivative blocks are spent)
+    if (tid + k * NT < ST::LO) ops[tid + k * NT] = low[k];
   __syncthreads();
   float gp[6] = {0, 0, 0, 0, 0, 0};   // d/dsigma_max[3], d/dp_sigma[3] (this thread's points)
   const int R = TE * 6;
@@ -515,6 +534,14 @@ sym_adj_kernel(const AdjParams<float> A,
       for (int g = part; g < ng; g += 2) {
         float w[4], o[4], su[4], sv[4], sw[4];
         sym_interp2<N, G, true>(C.p + g * CP, s, p, w, o);
+        if constexpr (ST::LO) {
+          sym_interp2<N, G, false>(ops + g * CP, s, p, su, sv);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            w[i] += su[i];
+            o[i] += sv[i];
+          }
+        }
         lds4(sg + g * 12 + u * 4, su);
         lds4(sg + g * 12 + v_ * 4, sv);
         lds4(sg + g * 12 + w_ * 4, sw);
