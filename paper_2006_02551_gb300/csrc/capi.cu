@@ -1986,10 +1986,12 @@ wadg_status wadg_memory_report(const wadg_ctx* ctx, size_t* bytes_state, size_t*
   if (bytes_pml_coeff)
     *bytes_pml_coeff = ctx->scheme == WADG_PML_STORED ? ctx->stored.bytes
                                                        : ctx->sig.bytes + ctx->kap.bytes;
-  if (bytes_operators) *bytes_operators = ctx->ops.bytes + ctx->tabs.bytes;
+  if (bytes_operators)
+    *bytes_operators = ctx->ops.bytes + ctx->tabs.bytes + ctx->tcops.bytes + ctx->symops.bytes +
+                       ctx->symadj.bytes + ctx->symtab.bytes + ctx->qslot.bytes;
   if (bytes_geometry)
     *bytes_geometry = ctx->geo.bytes + ctx->geof.bytes + ctx->fnrm.bytes + ctx->mat.bytes +
-                      ctx->nbr.bytes + ctx->code.bytes;
+                      ctx->nbr.bytes + ctx->code.bytes + ctx->facex.bytes + ctx->geox.bytes;
   return WADG_OK;
 }
 
@@ -2435,10 +2437,16 @@ wadg_status group_branches(wadg_group* g) {
   return WADG_OK;
 }
 
-// device bytes a member reads or writes in a step
+// device bytes a member reads or writes in a step: the symmetric stage reads
+// facex and geox, the tensor-core and the dense stages the tables they are made of
 size_t member_step_bytes(const wadg_ctx* x) {
-  return 2 * x->q[0].bytes + x->rq.bytes + x->p.bytes + x->rp.bytes + x->sig.bytes + x->kap.bytes +
-         x->geo.bytes + x->fnrm.bytes + x->mat.bytes + x->nbr.bytes + x->code.bytes;
+  const size_t state = 2 * x->q[0].bytes + x->rq.bytes + x->p.bytes + x->rp.bytes;
+  const size_t pml = x->sig.bytes + x->kap.bytes + x->stored.bytes;
+  const size_t tables = x->fnrm.bytes + x->mat.bytes + x->code.bytes;
+  if (x->tc) return state + pml + x->nbr.bytes + tables + (x->qc ? x->geof.bytes : x->geo.bytes);
+  const bool dense = x->K1 > 0 && (!x->sym.G || x->scheme == WADG_PML_STORED);
+  return state + pml + x->nbr.bytes + x->facex.bytes + x->geox.bytes +
+         (dense ? tables + x->geo.bytes : 0);
 }
 
 // members packed into clusters of at most half the L2 (smallest first);
