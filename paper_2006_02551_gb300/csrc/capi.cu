@@ -717,13 +717,15 @@ wadg_status upload_sources(wadg_ctx* ctx) {
       wk[i] = a / ctx->J_u[k];
       w.push_back((Real)wk[i]);
     }
-    for (double v : sym_adapt(ctx->N, wk)) ws.push_back((Real)v);
+    if (!ctx->tc)
+      for (double v : sym_adapt(ctx->N, wk)) ws.push_back((Real)v);
   }
   CK(dalloc(ctx->src, sd.size() * sizeof(SrcDev)));
   CK(dalloc(ctx->srcw, w.size() * sizeof(Real)));
   CK(dalloc(ctx->srcws, ws.size() * sizeof(Real)));
   if (!sd.empty()) {
-    CK(cudaMemcpy(ctx->srcws.p, ws.data(), ws.size() * sizeof(Real), cudaMemcpyHostToDevice));
+    if (!ws.empty())
+      CK(cudaMemcpy(ctx->srcws.p, ws.data(), ws.size() * sizeof(Real), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(ctx->src.p, sd.data(), sd.size() * sizeof(SrcDev), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(ctx->srcw.p, w.data(), w.size() * sizeof(Real), cudaMemcpyHostToDevice));
   }

@@ -634,14 +634,16 @@ sym_adj_kernel(const AdjParams<float> A,
     }
   }
   // source term of dJ/deps_k: + mu_E . J / eps^2
-  for (int s = sb0; s < sb1; ++s) {
+  // (a warp per source)
+  for (int s = sb0 + (tid >> 5); s < sb1; s += NT / 32) {
     const SrcDev& sd = A.src[s];
     const int e = sd.elem - eg0;
     const float ie = GX[e * 12 + 10];
     const float jt = (float)dipole_current(sd, A.t) * ie * ie;
-    for (int i = tid; i < 3 * Np; i += NT)
-      atomicAdd(&GE[e], jt * (float)sd.dir[i / Np] * A.src_w[(int64_t)s * Np + i % Np] *
-                            MQ[e * 6 * Np + i]);
+    float g = 0.f;
+    for (int i = tid & 31; i < 3 * Np; i += 32)
+      g += (float)sd.dir[i / Np] * A.src_w[(int64_t)s * Np + i % Np] * MQ[e * 6 * Np + i];
+    atomicAdd(&GE[e], jt * g);
   }
   // ---- lambda_in = lambda_out + dt L^T mu, rho_prev = A_i mu (all loads first)
   constexpr int UT = (ST::T * 3 * Np + NT - 1) / NT;

@@ -673,6 +673,7 @@ __device__ __forceinline__ bool sym_body(const StageParams<Real>& P, const SymCo
   const unsigned char* t_or = tab + 8 * Nfp;      // node orbits
   const unsigned char* fperm = tab + ST::TAB + NF;
   __shared__ int nsl, src0, dyn_tile;   // the tile's sources: count, first of the table
+  __shared__ Real cur[32];
   const int tid = threadIdx.x;
 
   for (int i = tid; i < ST::ops / 2; i += NT) {
@@ -1002,11 +1003,18 @@ __device__ __forceinline__ bool sym_body(const StageParams<Real>& P, const SymCo
     }
     const int sb0 = src0, sb1 = sb0 + nsl;
     __syncthreads();
-    if (sb1 > sb0) {   // dipole sources: adapted coefficients of M_k^-1 l(r_s)
-      for (int s = sb0; s < sb1; ++s) {   // (a thread keeps its values of an element)
+    // dipole sources: adapted coefficients of M_k^-1 l(r_s), the currents (in
+    // double) of 32 sources at a time by as many threads
+    for (int s0 = sb0; s0 < sb1; s0 += 32) {
+      if (tid < 32 && s0 + tid < sb1) {
+        const SrcDev& sd = P.src[s0 + tid];
+        cur[tid] = (Real)dipole_current(sd, tst) * GX[(sd.elem - eg0) * 12 + 10];
+      }
+      __syncthreads();
+      for (int s = s0; s < min(sb1, s0 + 32); ++s) {   // (a thread keeps its values of an element)
         const SrcDev& sd = P.src[s];
         const int e = sd.elem - eg0;
-        const Real jt = (Real)dipole_current(sd, tst) * GX[e * 12 + 10];
+        const Real jt = cur[s - s0];
         for (int i = tid; i < 3 * Np; i += NT) {
           const int c = i / Np;
           U[e * 2 * UST + i] -= jt * (Real)sd.dir[c] * P.src_ws[(int64_t)s * Np + i - c * Np];

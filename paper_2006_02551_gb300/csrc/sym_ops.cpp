@@ -252,16 +252,11 @@ std::vector<float> sym_transposed(int N, const std::vector<double>& ops) {
 }
 
 std::vector<double> sym_adapt(int N, const std::vector<double>& f) {
-  std::vector<Signed> T;
-  switch (N) {
-    case 1: T = node_sums_v4<1>(); break;
-    case 2: T = node_sums_v4<2>(); break;
-    case 3: T = node_sums_v4<3>(); break;
-    case 4: T = node_sums_v4<4>(); break;
-    default: T = node_sums_v4<5>(); break;
-  }
+  static const std::vector<Signed> sums[] = {{}, node_sums_v4<1>(), node_sums_v4<2>(),
+                                             node_sums_v4<3>(), node_sums_v4<4>(),
+                                             node_sums_v4<5>()};
   std::vector<double> t;
-  for (const Signed& s : T) {
+  for (const Signed& s : sums[N]) {
     double v = 0.0;
     for (const auto& p : s) v += p.second * f[p.first];
     t.push_back(v / (double)s.size());
