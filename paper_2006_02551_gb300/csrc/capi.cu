@@ -844,27 +844,33 @@ cudaError_t launch_pml_class(wadg_ctx* ctx, const StageParams<Real>& P) {
   return launch_pml_class<Real>(ctx, P, ctx->stream);
 }
 
-// the non-PML class of a stage on stream s (the kernel of the context's kind)
+// the non-PML class of a stage on stream s (the kernel of the context's kind);
+// branch: the PML class is launched beside it, on another stream
 template <typename Real>
-cudaError_t launch_std_class(wadg_ctx* ctx, const StageParams<Real>& P, cudaStream_t s) {
+cudaError_t launch_std_class(wadg_ctx* ctx, const StageParams<Real>& P, cudaStream_t s,
+                             bool branch = false) {
   if constexpr (std::is_same<Real, float>::value)
     if (ctx->tc) return launch_tc_rows(ctx->N, false, P, ctx->nb, s, ctx->bf16);
-  return launch_sym<Real>(ctx->N, 0, false, P, nullptr, ctx->nb, s);
+  const bool dense = !ctx->sym.G || ctx->scheme == WADG_PML_STORED;
+  const DensePml beside = !branch || !dense || ctx->K1 == 0 ? DensePml::none
+                          : ctx->K1 >= ctx->K0              ? DensePml::longer
+                                                            : DensePml::shorter;
+  return launch_sym<Real>(ctx->N, 0, false, P, nullptr, ctx->nb, s, beside);
 }
 
 // one element class of one stage of a context, on stream s, with the device
 // clock (graph replays); tile: elements per tile of the CUDA-core kernels
 // (0: the largest)
 cudaError_t launch_member_class(wadg_ctx* x, int st, double dt, bool pml, int tile,
-                                cudaStream_t s) {
+                                cudaStream_t s, bool branch) {
   if (x->rs == 8) {
     StageParams<double> P = stage_params<double>(x, st, dt, 0.0, true, pml);
     P.tile_elems = tile;
-    return pml ? launch_pml_class<double>(x, P, s) : launch_std_class<double>(x, P, s);
+    return pml ? launch_pml_class<double>(x, P, s) : launch_std_class<double>(x, P, s, branch);
   }
   StageParams<float> P = stage_params<float>(x, st, dt, 0.0, true, pml);
   P.tile_elems = x->tc ? 0 : tile;
-  return pml ? launch_pml_class<float>(x, P, s) : launch_std_class<float>(x, P, s);
+  return pml ? launch_pml_class<float>(x, P, s) : launch_std_class<float>(x, P, s, branch);
 }
 
 template <typename Real>
@@ -906,7 +912,7 @@ wadg_status issue_stage_branches(wadg_ctx* ctx, int stage, double dt) {
     StageParams<Real> B = stage_params<Real>(ctx, stage, dt, 0.0, true, true);
     CK(launch_pml_class<Real>(ctx, B));
     StageParams<Real> A = stage_params<Real>(ctx, stage, dt, 0.0, true, false);
-    CK(launch_std_class<Real>(ctx, A, ctx->aux));
+    CK(launch_std_class<Real>(ctx, A, ctx->aux, true));
   }
   CK(cudaEventRecord(ctx->ev_join, ctx->aux));
   CK(cudaStreamWaitEvent(ctx->stream, ctx->ev_join, 0));
@@ -2553,7 +2559,7 @@ cudaError_t group_launch_items(wadg_group* g, int par, int st) {
     // the buffers of this parity and stage (each stage flips them, a step once)
     const int cur0 = x->cur;
     x->cur = cur0 ^ par ^ (st & 1);
-    e = launch_member_class(x, st, g->dt_now[it.c], it.pml, it.tile, s);
+    e = launch_member_class(x, st, g->dt_now[it.c], it.pml, it.tile, s, nbr > 1);
     x->cur = cur0;
     if (e != cudaSuccess) return e;
   }

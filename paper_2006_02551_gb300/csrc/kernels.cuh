@@ -195,12 +195,16 @@ cudaError_t launch_stage(int N, bool kappa, const StageParams<Real>& P, int nb, 
                          int qc = 0);
 // the symmetric stage: G = 0 the non-PML class, 4 or 2 the PML class with a
 // volume rule of that symmetry (SymRule); coef: the rule's FP32 coefficients in
-// host memory (V_q, then P_q, ngroups x sym_cp(N, G) each), read by the call
+// host memory (V_q, then P_q, ngroups x sym_cp(N, G) each), read by the call;
+// beside: for the non-PML class, whether its PML class has the dense stage, and
+// whether that takes longer
+enum class DensePml { none, shorter, longer };
 template <typename Real>
 cudaError_t configure_sym_kernels(int N);
 template <typename Real>
 cudaError_t launch_sym(int N, int G, bool kappa, const StageParams<Real>& P, const float* coef,
-                       int nb, cudaStream_t s);
+                       int nb, cudaStream_t s,
+                       DensePml beside = DensePml::none);
 // both classes of a stage (A: non-PML, B: PML) in one launch, where their tiles
 // fit one wave of blocks (*done: whether it was launched).  chained: the launch
 // follows the last stage's on the stream, and may set its tables up before that

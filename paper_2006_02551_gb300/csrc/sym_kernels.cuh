@@ -39,12 +39,13 @@ cudaError_t sym_configure_one() {
   cudaError_t e = cudaFuncSetAttribute(sym_stage_kernel<Real, N, G, KAPPA>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)ST::max_bytes());
-  // the driver's own choice left room for two of three blocks
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(sym_stage_kernel<Real, N, G, KAPPA>,
-                             cudaFuncAttributePreferredSharedMemoryCarveout,
-                             cudaSharedmemCarveoutMaxShared);
   if constexpr (ST::PML) {
+    // the driver's own choice left room for two of three blocks (the non-PML
+    // class asks for it per launch: sym_launch_one)
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(sym_stage_kernel<Real, N, G, KAPPA>,
+                               cudaFuncAttributePreferredSharedMemoryCarveout,
+                               cudaSharedmemCarveoutMaxShared);
     constexpr size_t other = SymTile<Real, N, 0>::max_bytes();
     const size_t most = ST::max_bytes() > other ? ST::max_bytes() : other;
     if (e == cudaSuccess)
@@ -98,7 +99,7 @@ inline int sym_tile64(int tmax, int rows, int64_t n) {
 
 template <typename Real, int N, int G, bool KAPPA>
 cudaError_t sym_launch_one(const StageParams<Real>& P, const float* coef, int nb,
-                           cudaStream_t s) {
+                           cudaStream_t s, DensePml beside) {
   using ST = SymTile<Real, N, G, KAPPA>;
   if (P.n_elem <= 0) return cudaSuccess;
   StageParams<Real> Q = P;
@@ -114,7 +115,10 @@ cudaError_t sym_launch_one(const StageParams<Real>& P, const float* coef, int nb
   int per_sm = 1;
   cudaError_t e = resident(ST::tile_max(S), &per_sm);
   if (e != cudaSuccess) return e;
-  int te = sizeof(Real) == 8 && ST::PML
+  // beside a dense PML launch that takes longer: as few blocks as do it, since
+  // they only have to end before the other's (and each one delays a block of it)
+  int te = beside == DensePml::longer ? ST::tile_max(S)
+           : sizeof(Real) == 8 && ST::PML
                ? sym_tile64(ST::tile_max(S), 12 * S, (int64_t)P.n_elem * nb)
                : sym_tile(ST::tile_max(S), (int64_t)P.n_elem * nb, per_sm * sm_count());
   if (P.tile_elems > 0 && P.tile_elems < te) te = P.tile_elems;
@@ -124,8 +128,20 @@ cudaError_t sym_launch_one(const StageParams<Real>& P, const float* coef, int nb
   const long long tiles = (long long)((P.n_elem + te - 1) / te) * nb;
   const int grid = (int)std::min<long long>(tiles, (long long)per_sm * sm_count());
   const auto C = sym_coef<ST>(coef, P.ngroups);
-  sym_stage_kernel<Real, N, G, KAPPA><<<grid, ST::NT, smem, s>>>(Q, C);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(ST::NT);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  // room for several blocks, except beside a dense PML launch, which reads its
+  // operators through L1 and would lose that on every SM (stored scheme, N = 3,
+  // 24,576 tets, a stage: 170 us without this preference, 196 with it)
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+  at.val.sharedMemCarveout = cudaSharedmemCarveoutMaxShared;
+  cfg.attrs = &at;
+  cfg.numAttrs = ST::PML || beside != DensePml::none ? 0 : 1;
+  return cudaLaunchKernelEx(&cfg, sym_stage_kernel<Real, N, G, KAPPA>, Q, C);
 }
 
 template <typename Real, int N, int G, bool KAPPA>
@@ -197,13 +213,13 @@ cudaError_t sym_configure_n() {
 
 template <typename Real, int N>
 cudaError_t sym_launch_n(int G, bool kappa, const StageParams<Real>& P, const float* coef, int nb,
-                         cudaStream_t s) {
-  if (G == 0) return sym_launch_one<Real, N, 0, false>(P, coef, nb, s);
+                         cudaStream_t s, DensePml beside) {
+  if (G == 0) return sym_launch_one<Real, N, 0, false>(P, coef, nb, s, beside);
   if (G == 2)
-    return kappa ? sym_launch_one<Real, N, 2, true>(P, coef, nb, s)
-                 : sym_launch_one<Real, N, 2, false>(P, coef, nb, s);
-  return kappa ? sym_launch_one<Real, N, 4, true>(P, coef, nb, s)
-               : sym_launch_one<Real, N, 4, false>(P, coef, nb, s);
+    return kappa ? sym_launch_one<Real, N, 2, true>(P, coef, nb, s, beside)
+                 : sym_launch_one<Real, N, 2, false>(P, coef, nb, s, beside);
+  return kappa ? sym_launch_one<Real, N, 4, true>(P, coef, nb, s, beside)
+               : sym_launch_one<Real, N, 4, false>(P, coef, nb, s, beside);
 }
 
 template <typename Real, int N, int G, bool KAPPA>
@@ -238,9 +254,9 @@ int sym_split_n(int G, bool kappa, int64_t n) {
   }                                                                                     \
   template <>                                                                           \
   cudaError_t launch_sym<Real>(int N, int G, bool kappa, const StageParams<Real>& P,    \
-                               const float* coef, int nb, cudaStream_t s) {             \
+                               const float* coef, int nb, cudaStream_t s, DensePml beside) { \
     auto f = [&](auto n) {                                                              \
-      return sym_launch_n<Real, decltype(n)::value>(G, kappa, P, coef, nb, s);          \
+      return sym_launch_n<Real, decltype(n)::value>(G, kappa, P, coef, nb, s, beside);  \
     };                                                                                  \
     WADG_SYM_SWITCH(WADG_SYM_CALL)                                                      \
     return cudaErrorInvalidValue;                                                       \
