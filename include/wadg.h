@@ -428,8 +428,11 @@ wadg_status wadg_group_autotune(wadg_group* g, const double* dt, int32_t reps, d
  * parallel (1: a stage's launches on parallel branches), share (1: each
  * variant's grid its share of the GPU), tile_divisor (1..64), blocks_per_sm
  * (1..8, capped by each variant's occupancy).  EINVAL out of range;
- * EUNSUPPORTED for per_item = 0 in a group whose members the grouped variant
- * kernels do not serve. */
+ * EUNSUPPORTED for per_item = 0 in a group with members that the grouped variant
+ * kernels do not serve (another precision than FP32, a compact rule, the
+ * stored scheme).  Where members of one order have different volume rules, or a
+ * rule without the default one's symmetry, per_item = 0 is accepted and every
+ * item is launched on its own all the same (wadg_group_info: per_item = 1). */
 wadg_status wadg_group_set_tuning(wadg_group* g, int32_t per_item, int32_t parallel,
                                   int32_t share, int32_t tile_divisor, int32_t blocks_per_sm);
 
