@@ -636,6 +636,45 @@ __device__ __forceinline__ void sym_to_sums(Real* s) {
           j < B::NFul ? Real(4) : (x == 0 && j == 3 * B::NH + B::NFul ? Real(1) : Real(2));
 }
 
+// Dipole sources of a tile (s0 .. s1 of the table): the currents of the first 32
+// from s0 on by one warp, in double, scaled by 1/eps; and all of them, adapted
+// coefficients of M_k^-1 l(r_s), into the adapted right-hand sides U.  Every thread
+// evaluating every current took 2 us a source; in FP32 a warp that has no part in
+// the curl evaluates them meanwhile (evaluated after it, one source prolonged the
+// stage: kappa = 2, 29,478 tets, 10 steps 7.53 against 7.42 ms).  Not inlined: few
+// tiles have sources, and the others fetch less code.
+template <typename Real>
+__device__ __noinline__ void sym_currents(const SrcDev* src, int s0, int s1, int eg0, double t,
+                                          const Real* GX, Real* cur) {
+  const int k = threadIdx.x & 31;
+  if (s0 + k < s1) {
+    const SrcDev& sd = src[s0 + k];
+    cur[k] = (Real)dipole_current(sd, t) * GX[(sd.elem - eg0) * 12 + 10];
+  }
+}
+// (the first 32 currents are there)
+template <typename Real, int Np, int UST, int NT>
+__device__ __noinline__ void sym_sources(const SrcDev* src, const Real* src_ws, int s0, int s1,
+                                         int eg0, double t, const Real* GX, Real* cur, Real* U) {
+  const int tid = threadIdx.x;
+  for (int sb = s0; sb < s1; sb += 32) {
+    if (sb > s0) {
+      if (tid < 32) sym_currents(src, sb, s1, eg0, t, GX, cur);
+      __syncthreads();
+    }
+    for (int s = sb; s < min(s1, sb + 32); ++s) {   // (a thread keeps its values of an element)
+      const SrcDev& sd = src[s];
+      const int e = sd.elem - eg0;
+      const Real jt = cur[s - sb];
+      for (int i = tid; i < 3 * Np; i += NT) {
+        const int c = i / Np;
+        U[e * 2 * UST + i] -= jt * (Real)sd.dir[c] * src_ws[(int64_t)s * Np + i - c * Np];
+      }
+    }
+    __syncthreads();
+  }
+}
+
 // One element class of one context; smem_raw is the block's dynamic shared
 // memory.  Tiles by a static schedule, or from the counter *dyn (grouped
 // launch).  False where a copy did not land in time: the block then takes no
@@ -955,12 +994,14 @@ __device__ __forceinline__ bool sym_body(const StageParams<Real>& P, const SymCo
     }
     __syncthreads();
 
+    const int sb0 = src0, sb1 = sb0 + nsl;   // the tile's sources
     // ---- curl and LIFT in adapted values; results stay in registers until
     // every thread has read U, which then holds them: [TE][E, H][3][Np]
     // FP64: one row per task (the FP64 pipe bounds it, so the finest split
     // balances best); FP32: all rows of a character, for fewer loads per
     // multiplication, one character per warp
     if constexpr (sizeof(Real) == 8) {
+      if (sb1 > sb0 && tid < 32) sym_currents(P.src, sb0, sb1, eg0, tst, GX, cur);
       constexpr int MT = (ST::T * 2 * Np + NT - 1) / NT;
       Real res[MT][3];
 #pragma unroll
@@ -984,16 +1025,18 @@ __device__ __forceinline__ bool sym_body(const StageParams<Real>& P, const SymCo
         for (int c = 0; c < 3; ++c) U[(ef ^ 1) * UST + c * Np + row] = res[k][c];
       }
     } else {
-      // warps 0-3 and 4-7: characters 0-3 of the first 32 rows and the others
-      const int x = (tid >> 5) & 3, ef = (tid >> 7) * 32 + (tid & 31), f = ef & 1;
-      const bool act = ef < 2 * ne;
+      // warps 0-3: characters 0-3, a lane per (element, field)
+      static_assert(2 * ST::T <= 32, "a warp holds the tile's rows of a character");
+      const int x = (tid >> 5) & 3, ef = tid & 31, f = ef & 1;
+      const bool act = tid < 128 && ef < 2 * ne;
       const int r = act ? ef : 0;   // spare lanes repeat row 0 and write nothing
       const Real* g = GX + (r >> 1) * 12;
       const Real sc = f ? g[10] : -g[11];
       Real* out = act ? U + (ef ^ 1) * UST : nullptr;
       const Real* uu = U + r * UST;
       const Real* ff = FL + (r ^ 1) * FST;
-      if ((ef & ~31) >= 2 * ne) {   // no row of this warp's
+      if (tid >= 128) {
+        if (sb1 > sb0 && tid < 160) sym_currents(P.src, sb0, sb1, eg0, tst, GX, cur);
         __syncthreads();
       } else if (x == 0) {
         sym_curl_pairs<N, 0, ST::CC>(ops, 0, uu, ff, g, sc, out);
@@ -1001,27 +1044,9 @@ __device__ __forceinline__ bool sym_body(const StageParams<Real>& P, const SymCo
         sym_curl_pairs<N, 1, ST::CC>(ops, x, uu, ff, g, sc, out);
       }
     }
-    const int sb0 = src0, sb1 = sb0 + nsl;
     __syncthreads();
-    // dipole sources: adapted coefficients of M_k^-1 l(r_s), the currents (in
-    // double) of 32 sources at a time by as many threads
-    for (int s0 = sb0; s0 < sb1; s0 += 32) {
-      if (tid < 32 && s0 + tid < sb1) {
-        const SrcDev& sd = P.src[s0 + tid];
-        cur[tid] = (Real)dipole_current(sd, tst) * GX[(sd.elem - eg0) * 12 + 10];
-      }
-      __syncthreads();
-      for (int s = s0; s < min(sb1, s0 + 32); ++s) {   // (a thread keeps its values of an element)
-        const SrcDev& sd = P.src[s];
-        const int e = sd.elem - eg0;
-        const Real jt = cur[s - s0];
-        for (int i = tid; i < 3 * Np; i += NT) {
-          const int c = i / Np;
-          U[e * 2 * UST + i] -= jt * (Real)sd.dir[c] * P.src_ws[(int64_t)s * Np + i - c * Np];
-        }
-      }
-      __syncthreads();
-    }
+    if (sb1 > sb0)
+      sym_sources<Real, Np, UST, NT>(P.src, P.src_ws, sb0, sb1, eg0, tst, GX, cur, U);
 
     if constexpr (!PML) {
       // ---- back to nodal values, in place
