@@ -115,8 +115,9 @@ __device__ __forceinline__ void lds2(const double* p, double* v) {
 }
 
 // Stage kernel.  Threads work on register tiles: 4 nodes x 3 components x 3
-// reference derivatives (curl), 4 quadrature points x 12 components (V_q),
-// smem_raw is the block's dynamic shared memory; block `bid` of `nblk` takes
+// reference derivatives (curl), 4 quadrature points x 12 components (V_q), 4
+// nodes x 4 components (P_q); all operator reads come from shared memory where
+// the operators fit it.  smem_raw is the block's dynamic shared memory; block `bid` of `nblk` takes
 // tiles bid, bid + nblk, ...
 template <typename Real, int N, bool KAPPA, bool STORED, int QC = 0>
 __device__ __forceinline__ void stage_body(const StageParams<Real>& P, unsigned char* smem_raw,
@@ -132,7 +133,7 @@ __device__ __forceinline__ void stage_body(const StageParams<Real>& P, unsigned 
   const Real* DtT = DsT + Np * NpP;
   const Real* LIFTT = DtT + Np * NpP;
   const Real* VqT = LIFTT + NF * NpP;
-  const Real* PqT = VqT + Np * NqP;  
+  const Real* PqT = VqT + Np * NqP;
   // elements per tile: T, or fewer when the launch asks for smaller tiles
   // (the shared-memory carve-up follows, so smaller tiles need less of it)
   const int TE = P.tile_elems > 0 && P.tile_elems < T ? P.tile_elems : T;

@@ -34,7 +34,7 @@
 namespace wadg {
 namespace tc {
 
-// Shared-memory plan of one tile (all offsets in bytes).  
+// Shared-memory plan of one tile (all offsets in bytes).
 template <int N, bool BF>
 struct Plan {
   using O = OpT<BF>;

@@ -2,8 +2,9 @@
 // TF32 or BF16 operands, FP32 accumulation in tensor memory, FP32 state) for
 // the non-PML class (PML = false drops the P rows, V_q, P_q and eq. 9) and for
 // the PML class of contexts with a compact volume rule (quad_capacity class
-// 1).  The PML class with the (N+1)^3 rule runs tc_stage_kernel: its points do
-// not fit the tensor memory of row-owned products.
+// 1), whose capacity the plan below is made for.  The PML class with the (N+1)^3
+// rule runs tc_stage_kernel; a plan with that rule's points (two slots at N <= 3,
+// one at N = 4 by its tensor-memory columns) has not been built or measured.
 //
 // What bounds it: the chain of a tile (operands -> V_q -> eq. 9 -> P_q ->
 // update, the curl between) in the epilogue warps, and the flux warps beside
