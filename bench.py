@@ -40,8 +40,8 @@ import numpy as np  # noqa: E402
 # the kernel source it was taken on (sha256 of that source file): None until
 # a capture of the current source is recorded here
 TC_PML_TRAFFIC = {"file": "tc_rows.cu",
-                  "sha256": "03c2281bf80d113027f62a6bcb2b664322eb0a8f8f618bf49652a5f58d3a1592",
-                  "N": 4, "bytes_per_pml_element": {"tf32": 6333.3, "bf16": 6336.2}}
+                  "sha256": "9a7cd34548a0c76099d46eb08cd637d782c0be744b11550db66d7368b4fabcfb",
+                  "N": 4, "bytes_per_pml_element": {"tf32": 6268.9, "bf16": 6269.2}}
 
 
 def tc_pml_traffic(K1, N, precision):
@@ -85,6 +85,28 @@ def algorithmic_costs(N, Np, Nfp, Nq, rs, kappa, rows=False):
     if kappa:
         f_pml += 24 * Nq * Np + 6 * Nq
     return dict(bytes_std=b_std, bytes_pml=b_pml, flops_std=f_std, flops_pml=f_pml)
+
+
+def block_flops(N, Np, Nfp, groups, G, kappa, fp64):
+    """Flops per element of a stage launch of the symmetric CUDA-core stage:
+    (non-PML, PML).  The reference operators act on symmetry-adapted values: the
+    nodes' orbits under the group of four vertex permutations give D0 values of
+    its first character and D1 of each other; d/dxi_a takes block x to x xor a and
+    LIFT is block diagonal.  groups, G: the volume rule's groups of four points
+    and its symmetry (4: one orbit a group; 2: two)."""
+    fixed = N // 2 + 1 if N % 2 == 0 else 0          # nodes that one permutation fixes
+    D0, D1 = (Np + 3 * fixed) // 4, (Np - fixed) // 4
+    D = 6 * D0 * D1 + 6 * D1 * D1                     # coefficients of the three derivatives
+    # both fields: FP32 three derivatives a component, FP64 two (covariant curl);
+    # then the metric, LIFT, two additions per value of each butterfly (fields in
+    # and out, flux), the flux at 4 Nfp nodes and the update
+    f = (8 if fp64 else 12) * D + (36 if fp64 else 72) * Np + 12 * Nfp * Np
+    f += 24 * Np + 48 * Nfp + 240 * Nfp + 24 * Np
+    coefs = 4 // G * Np * groups                      # of V_q, and of P_q
+    g = f + 48 * coefs + 24 * 4 * groups + 36 * Np + 48 * Np + 96 * 2 * groups
+    if kappa:
+        g += 24 * coefs + 24 * groups + 24 * Np
+    return f, g
 
 
 class ClockSampler:
@@ -670,8 +692,14 @@ def main():
         peak = fma_peak(local, fp64=args.precision == "fp64")
         peak_note = (f"measured {'FP64' if args.precision == 'fp64' else 'FP32'} FMA "
                      f"throughput (wadg_fma_peak: register FMA chains on every SM)")
+        kap = w.pml.kappa_max != 1.0
+        bf = block_flops(N, Np, Nfp, nq_read / (8 if kap else 4), 4 if args.rule == "compact" else 2,
+                         kap, args.precision == "fp64")
+        d_flops = (bf[1] * K1 if dom == "pml" else bf[0] * (K - K1)) * w.n_batch
+        dense, achieved = achieved, d_flops / (d_ms * 1e-3) / 1e12
         roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                     "frac": achieved / peak, "traffic": None, "kernel": f"sym_stage_kernel<{dom}>",
+                    "dense_equivalent_tflops": dense,
                     "peak_source": peak_note,
                     "hbm": {"achieved_gbs": achieved_gbs, "peak_gbs": hbm,
                             "frac": achieved_gbs / hbm}}
@@ -719,8 +747,13 @@ def main():
             so.set_state(None, 0.0)
             so.run_steps(nst, dt, record=False)
             qo, _ = so.get_state()
+            # groups of four samples (three axes, and as many kappa samples) per element
+            groups = so.memory_report()["pml_coeff"] / max(1, K1) / (8 if prec == "fp64" else 4) / (
+                24 if w.pml.kappa_max != 1.0 else 12)
             so.close()
             others[prec] = ({"value": dofs / (mso * 1e-3), "ms_per_step": mso}, qo)
+            if prec in ("fp32", "fp64"):
+                others[prec][0]["groups"] = groups
         sel = (slice(None), slice(None), slice(0, 6))
         if "fp64" in others:
             q64 = others["fp64"][1]
@@ -744,13 +777,17 @@ def main():
         out_extra["cuda_core_peaks_tflops"] = peaks_fma
         for prec in ("fp32", "fp64"):
             if prec in out_extra:
-                c2 = algorithmic_costs(N, Np, Nfp, Nq, 8 if prec == "fp64" else 4,
-                                       w.pml.kappa_max != 1.0)
-                fl = 5 * (c2["flops_std"] * (K - K1) + c2["flops_pml"] * K1) * w.n_batch
-                ach = fl / (out_extra[prec]["ms_per_step"] * 1e-3) / 1e12
-                out_extra[prec]["alu"] = {"achieved_tflops": ach, "peak_tflops": peaks_fma[prec],
-                                          "frac": ach / peaks_fma[prec],
-                                          "peak_source": "measured FMA throughput"}
+                kap = w.pml.kappa_max != 1.0
+                c2 = algorithmic_costs(N, Np, Nfp, Nq, 8 if prec == "fp64" else 4, kap)
+                bf = block_flops(N, Np, Nfp, out_extra[prec].pop("groups"),
+                                 4 if args.rule == "compact" else 2, kap, prec == "fp64")
+                per_s = 5 * w.n_batch / (out_extra[prec]["ms_per_step"] * 1e-3) / 1e12
+                ach = per_s * (bf[0] * (K - K1) + bf[1] * K1)
+                out_extra[prec]["alu"] = {
+                    "achieved_tflops": ach, "peak_tflops": peaks_fma[prec],
+                    "frac": ach / peaks_fma[prec], "peak_source": "measured FMA throughput",
+                    "dense_equivalent_tflops":
+                        per_s * (c2["flops_std"] * (K - K1) + c2["flops_pml"] * K1)}
     else:
         s.close()
 
