@@ -37,8 +37,9 @@ struct SaTile {
   // a mesh in the profile derivatives: median relative error of dJ/dsigma_max, N =
   // 4, 16,464 tets, 8.3e-7 without the low parts, 3.8e-7 with them, 3.3e-7 in the
   // dense kernel with its 48 times 35 coefficients (N = 5, 6,000 tets: 3.3e-6,
-  // 2.3e-6, 2.3e-6).  A gradient takes 1.2 % longer for them (N = 3, 82,944 tets).  Z2 rules have
-  // several times as many coefficients and the dense kernel's errors.
+  // 2.3e-6, 2.3e-6).  A gradient takes 1.2 % longer for them (N = 3, 82,944
+  // tets, 40 steps: 129.9 -> 131.5 ms).  Z2 rules have several times as many
+  // coefficients and the dense kernel's errors.
   static constexpr int LO = G == 4 ? NG * CP : 0, LOT = (LO + kSaThreads - 1) / kSaThreads;
   static_assert(LO <= DT, "low parts of P_q");
   static constexpr int TAB = 8 * Nfp + 4 * B::NFul + 8 + 3 * Np;
